@@ -116,7 +116,7 @@ int launch_coarse64(const ModelDev& m, int n, double h, double* u, const double*
                     const double* S, int sweeps, cudaStream_t st);
 int launch_residual_restrict64(const ModelDev& m, int nf, double hf, const double* u,
                                const double* rho, const double* S, double* Ru, double* uH,
-                               double* Rd, cudaStream_t st);
+                               double* Rd, bool relaxed, cudaStream_t st);
 int launch_fas_source64(const ModelDev& m, int nc, double hc, const double* Ru,
                         const double* rho, double* S, cudaStream_t st);
 int launch_density_mean(const float* rho32, size_t n3, double* partials, double* out_sum,

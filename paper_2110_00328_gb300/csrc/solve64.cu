@@ -11,95 +11,66 @@
 
 #include <chrono>
 
+#include "fp64_fast.cuh"
 #include "mg_common.cuh"
 #include "mg_internal.h"
 
 namespace mg {
 
 // ---------------------------------------------------------------------------
-// Device arithmetic of one cell
+// Kernels
 // ---------------------------------------------------------------------------
+//
+// All of them are bound by the FP64 pipe (fp64_fast.cuh), not by memory: at 96^3
+// a colour pass reads 21 MB, 3 us from HBM, and issues 15 FP64 instructions a
+// cell, 11 us at 0.58e12 a second.  So the work is laid out to spend few of
+// those: products folded into the sums, one reciprocal a cell, transfers that
+// share their partial sums, and nothing formed that is known.
+
+// Threads of the 3D kernels: 16 cells along k by 16 rows j of one plane i.  Rows
+// of 48 or 80 cells fill them, which 64 threads along k did not.
+constexpr int kTx = 16, kTy = 16;
+#define MG_CELL3(nk, nj)                              \
+  const int k = blockIdx.x * kTx + threadIdx.x;       \
+  const int j = blockIdx.y * kTy + threadIdx.y;       \
+  const int i = blockIdx.z;                           \
+  if (k >= (nk) || j >= (nj)) return
 
 // Sum over the six face neighbours of the field that enters the Laplacian
-// (f(R): w = u^{n+1}; symmetron, CQ: u itself).
+// (f(R): w = u^{n+1}; symmetron, CQ: u itself), the power folded into the sum.
 template <int K>
-__device__ __forceinline__ double nb_sum64(const double* __restrict__ u, int n, int i, int j, int k) {
+__device__ __forceinline__ double nb_sum64(const double* u, int n, int i, int j, int k) {
   const int ip = wrapi(i + 1, n), im = wrapi(i - 1, n);
   const int jp = wrapi(j + 1, n), jm = wrapi(j - 1, n);
   const int kp = wrapi(k + 1, n), km = wrapi(k - 1, n);
-  return fr_or_id<K>(u[cidx(n, ip, j, k)]) + fr_or_id<K>(u[cidx(n, im, j, k)]) +
-         fr_or_id<K>(u[cidx(n, i, jp, k)]) + fr_or_id<K>(u[cidx(n, i, jm, k)]) +
-         fr_or_id<K>(u[cidx(n, i, j, kp)]) + fr_or_id<K>(u[cidx(n, i, j, km)]);
-}
-
-// N_h(u) at one cell (see mg_model.cuh for the three operators).
-template <int K>
-__device__ __forceinline__ double local_N64(const ModelDev& m, double h, double uc, double rhoc,
-                                            double Lnb) {
-  const double ih2 = 1.0 / (h * h);
-  if constexpr (is_fr(K)) {
-    const double w = fr_w<K>(uc);
-    return -m.c2 * (Lnb - 6.0 * w) * ih2 + m.om_a * (rhoc - 1.0) + m.K0 - m.K / uc;
-  } else if constexpr (K == KSYM) {
-    return m.c2 * (Lnb - 6.0 * uc) * ih2 - m.msym * ((rhoc * m.rat3 - 1.0) * uc + uc * uc * uc);
-  } else {
-    const double E = m.keep_exp ? exp(m.beta * uc / m.c2) : 1.0;
-    const double x = m.phibar + uc / m.c2;
-    return (Lnb - 6.0 * uc) * ih2 - m.cq_src * (E * rhoc - 1.0) +
-           m.cq_pot * (pow(x, -1.0 - m.alpha) - m.pot0);
+  const double v[6] = {u[cidx(n, ip, j, k)], u[cidx(n, im, j, k)], u[cidx(n, i, jp, k)],
+                       u[cidx(n, i, jm, k)], u[cidx(n, i, j, kp)], u[cidx(n, i, j, km)]};
+  double s = fr_or_id<K>(v[0]);
+#pragma unroll
+  for (int t = 1; t < 6; ++t) {
+    if constexpr (K == KFR1) s = fma(v[t], v[t], s);
+    else if constexpr (K == KFR2) s = fma(v[t] * v[t], v[t], s);
+    else s += v[t];
   }
+  return s;
 }
-
-// Gauss-Seidel update of one cell: the exact local root for f(R) and the
-// symmetron (nonlinear GS, Secs. 3.2.4-3.2.5), one Newton step for CQ
-// (Eq. relaxation_iteration, Sec. 3.2.3).  The FAS source S enters p (f(R))
-// or q (symmetron) of the local polynomial.
-template <int K>
-__device__ __forceinline__ double local_update64(const ModelDev& m, double h, double uc,
-                                                 double rhoc, double s, double Lnb) {
-  if constexpr (is_fr(K)) {
-    const double al = h * h / (6.0 * m.c2);
-    const double p = al * (m.om_a * (rhoc - 1.0) + m.K0 - s) - Lnb * (1.0 / 6.0);
-    const double q = -al * m.K;
-    return fr_root<K>(p, q);
-  } else if constexpr (K == KSYM) {
-    const double g = m.c2 * m.xi2_a2 / (h * h);
-    const double p = rhoc * m.rat3 - 1.0 + 12.0 * g;
-    const double q = -2.0 * g * Lnb + 2.0 * m.xi2_a2 * s;
-    return sym_root(p, q, uc);
-  } else {
-    const double ih2 = 1.0 / (h * h);
-    const double x = m.phibar + uc / m.c2;
-    const double E = m.keep_exp ? exp(m.beta * uc / m.c2) : 1.0;
-    const double dE = m.keep_exp ? (m.beta / m.c2) * E : 0.0;
-    const double px = pow(x, -1.0 - m.alpha);
-    const double r = (Lnb - 6.0 * uc) * ih2 - m.cq_src * (E * rhoc - 1.0) + m.cq_pot * (px - m.pot0) - s;
-    const double dr = -6.0 * ih2 - m.cq_src * dE * rhoc - m.cq_pot * (1.0 + m.alpha) * px / (x * m.c2);
-    return uc - r / dr;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Kernels
-// ---------------------------------------------------------------------------
 
 // Relax every cell of one colour ((i+j+k) % 2 == parity); one thread per cell.
+// Measured (f(R) n = 1): 15.6 us a pass at 96^3, 30.8 us at 128^3 (of that 11 and 26 us is the FP64
+// pipe); with cube root, square root and cosine in FP64 a 128^3 pass took 205 us.
 template <int K>
-__global__ void __launch_bounds__(kThreads) k_smooth64(ModelDev m, int n, double h, double* __restrict__ u,
-                                                       const double* __restrict__ rho,
+__global__ void __launch_bounds__(kTx* kTy) k_smooth64(Const64 c, int n, double* u, const double* __restrict__ rho,
                                                        const double* __restrict__ S, int parity) {
-  const int i = blockIdx.z, j = blockIdx.y;
-  const int kk = blockIdx.x * blockDim.x + threadIdx.x;
-  if (kk >= (n >> 1)) return;
-  const int k = 2 * kk + ((i + j + parity) & 1);
-  const size_t c = cidx(n, i, j, k);
-  const double Lnb = nb_sum64<K>(u, n, i, j, k);
-  u[c] = local_update64<K>(m, h, u[c], rho[c], S ? S[c] : 0.0, Lnb);
+  MG_CELL3(n >> 1, n);
+  const int kc = 2 * k + ((i + j + parity) & 1);
+  const size_t t = cidx(n, i, j, kc);
+  const double Lnb = nb_sum64<K>(u, n, i, j, kc);
+  u[t] = local_update64<K>(c, u[t], rho[t], S ? S[t] : 0.0, Lnb);
 }
 
 // d = N(u) - S on every cell; optional store of d; per-block partial sums of d^2.
 template <int K>
-__global__ void __launch_bounds__(kThreads) k_residual64(ModelDev m, int n, double h, const double* __restrict__ u,
+__global__ void __launch_bounds__(kThreads) k_residual64(Const64 c, int n, const double* __restrict__ u,
                                                          const double* __restrict__ rho,
                                                          const double* __restrict__ S, double* __restrict__ d,
                                                          double* __restrict__ partials) {
@@ -109,9 +80,10 @@ __global__ void __launch_bounds__(kThreads) k_residual64(ModelDev m, int n, doub
     const int i = r / n, j = r - (r / n) * n;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
       const size_t t = cidx(n, i, j, k);
-      const double v = local_N64<K>(m, h, u[t], rho[t], nb_sum64<K>(u, n, i, j, k)) - (S ? S[t] : 0.0);
+      const double N = local_N64<K>(c, u[t], rho[t], nb_sum64<K>(u, n, i, j, k));
+      const double v = S ? N - S[t] : N;
       if (d) d[t] = v;
-      acc += v * v;
+      acc = fma(v, v, acc);
     }
   }
   acc = block_sum(acc);
@@ -127,121 +99,145 @@ __global__ void k_finalize_sum(const double* __restrict__ partials, int count, d
 }
 
 // coarse = mean of the 8 children.
-__global__ void k_restrict64(int nf, const double* __restrict__ fine, double* __restrict__ coarse) {
+__global__ void __launch_bounds__(kTx* kTy) k_restrict64(int nf, const double* __restrict__ fine,
+                                                         double* __restrict__ coarse) {
   const int nc = nf >> 1;
-  const int I = blockIdx.z, J = blockIdx.y;
-  const int K = blockIdx.x * blockDim.x + threadIdx.x;
-  if (K >= nc) return;
+  MG_CELL3(nc, nc);
   double s = 0.0;
   for (int di = 0; di < 2; ++di)
     for (int dj = 0; dj < 2; ++dj)
-      for (int dk = 0; dk < 2; ++dk) s += fine[cidx(nf, 2 * I + di, 2 * J + dj, 2 * K + dk)];
-  coarse[cidx(nc, I, J, K)] = s * 0.125;
+      for (int dk = 0; dk < 2; ++dk) s += fine[cidx(nf, 2 * i + di, 2 * j + dj, 2 * k + dk)];
+  coarse[cidx(nc, i, j, k)] = s * 0.125;
 }
 
 // Fused: for each coarse cell, the local residual of its 8 children is formed
 // on the fly (the recomputation the paper also does, Sec. 3.2.2) and averaged
 // into Rd; the children's solution is averaged into Ru and copied to uH.
-template <int K>
-__global__ void __launch_bounds__(kThreads) k_residual_restrict64(ModelDev m, int nf, double hf,
-                                                                  const double* __restrict__ u,
+// ZR (f(R), symmetron, after pre-smoothing): the second colour ((i+j+k) odd) was
+// relaxed last, to the exact root of its own equation, so its residual is that
+// root's rounding; it is taken as zero and only the four first-colour children's
+// residuals are formed (as the mixed path does).
+template <int K, bool ZR>
+__global__ void __launch_bounds__(kTx* kTy) k_residual_restrict64(Const64 c, int nf, const double* __restrict__ u,
                                                                   const double* __restrict__ rho,
                                                                   const double* __restrict__ S,
                                                                   double* __restrict__ Ru, double* __restrict__ uH,
                                                                   double* __restrict__ Rd) {
+  static_assert(!ZR || K != KCQ, "CQ relaxes by one Newton step: its residual is not zero");
   const int nc = nf >> 1;
-  const int I = blockIdx.z, J = blockIdx.y;
-  const int K0 = blockIdx.x * blockDim.x + threadIdx.x;
-  if (K0 < nc) {
-    const size_t t = cidx(nc, I, J, K0);
-    double su = 0.0, sd = 0.0;
-    for (int di = 0; di < 2; ++di)
-      for (int dj = 0; dj < 2; ++dj)
-        for (int dk = 0; dk < 2; ++dk) {
-          const int i = 2 * I + di, j = 2 * J + dj, k = 2 * K0 + dk;
-          const size_t c = cidx(nf, i, j, k);
-          const double uc = u[c];
-          su += uc;
-          sd += local_N64<K>(m, hf, uc, rho[c], nb_sum64<K>(u, nf, i, j, k)) - (S ? S[c] : 0.0);
-        }
-    const double ru = su * 0.125;
-    Ru[t] = ru;
-    uH[t] = ru;
-    Rd[t] = sd * 0.125;
-  }
+  MG_CELL3(nc, nc);
+  double su = 0.0, sd = 0.0;
+#pragma unroll
+  for (int di = 0; di < 2; ++di)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj)
+#pragma unroll
+      for (int dk = 0; dk < 2; ++dk) {
+        const int a = 2 * i + di, b = 2 * j + dj, e = 2 * k + dk;
+        const size_t t = cidx(nf, a, b, e);
+        const double uc = u[t];
+        su += uc;
+        if (ZR && ((di + dj + dk) & 1)) continue;
+        const double N = local_N64<K>(c, uc, rho[t], nb_sum64<K>(u, nf, a, b, e));
+        sd += S ? N - S[t] : N;
+      }
+  const size_t t = cidx(nc, i, j, k);
+  const double ru = su * 0.125;
+  Ru[t] = ru;
+  uH[t] = ru;
+  Rd[t] = sd * 0.125;
 }
 
 // In place: S <- N^H(Ru) - S, where S holds R d on entry.
 template <int K>
-__global__ void __launch_bounds__(kThreads) k_fas_source64(ModelDev m, int n, double h, const double* __restrict__ Ru,
+__global__ void __launch_bounds__(kTx* kTy) k_fas_source64(Const64 c, int n, const double* __restrict__ Ru,
                                                            const double* __restrict__ rho, double* __restrict__ S) {
-  const int i = blockIdx.z, j = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
+  MG_CELL3(n, n);
   const size_t t = cidx(n, i, j, k);
-  S[t] = local_N64<K>(m, h, Ru[t], rho[t], nb_sum64<K>(Ru, n, i, j, k)) - S[t];
+  S[t] = local_N64<K>(c, Ru[t], rho[t], nb_sum64<K>(Ru, n, i, j, k)) - S[t];
 }
 
-// The prolongation weight stencil at fine cell (i,j,k) of coarse field c (side nc).
-__device__ __forceinline__ double prolong_at64(const double* __restrict__ c, int nc, int i, int j, int k) {
-  const int I = i >> 1, J = j >> 1, K = k >> 1;
-  const int I2 = wrapi(I + ((i & 1) ? 1 : -1), nc);
-  const int J2 = wrapi(J + ((j & 1) ? 1 : -1), nc);
-  const int K2 = wrapi(K + ((k & 1) ? 1 : -1), nc);
-  const double v = 27.0 * c[cidx(nc, I, J, K)] +
-                   9.0 * (c[cidx(nc, I2, J, K)] + c[cidx(nc, I, J2, K)] + c[cidx(nc, I, J, K2)]) +
-                   3.0 * (c[cidx(nc, I2, J2, K)] + c[cidx(nc, I2, J, K2)] + c[cidx(nc, I, J2, K2)]) +
-                   c[cidx(nc, I2, J2, K2)];
-  return v * (1.0 / 64.0);
-}
-
-// u^h += P(u^H - R u^h); f(R): non-positive results fall back to half the old value.
+// u^h += P(u^H - R u^h), the 27/9/3/1 (/64) weights; f(R): non-positive results
+// fall back to half the old value.  One thread per coarse cell, whose eight
+// children interpolate from the 27 coarse differences around it: the weights
+// factor into (3, 1) per axis, so the children share the sums along k and j (65
+// FP64 instructions for eight cells; a child at a time they are 152).
 template <bool FR>
-__global__ void __launch_bounds__(kThreads) k_prolong_correct64(int nc, const double* __restrict__ uH,
+__global__ void __launch_bounds__(kTx* kTy) k_prolong_correct64(int nc, const double* __restrict__ uH,
                                                                 const double* __restrict__ RuH,
                                                                 double* __restrict__ uf,
                                                                 unsigned long long* guard) {
+  MG_CELL3(nc, nc);
   const int nf = nc << 1;
-  const int i = blockIdx.z, j = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nf) {
-    const size_t t = cidx(nf, i, j, k);
-    const int I = i >> 1, J = j >> 1, K = k >> 1;
-    const int I2 = wrapi(I + ((i & 1) ? 1 : -1), nc);
-    const int J2 = wrapi(J + ((j & 1) ? 1 : -1), nc);
-    const int K2 = wrapi(K + ((k & 1) ? 1 : -1), nc);
-#define EH(a, b, c) (uH[cidx(nc, a, b, c)] - RuH[cidx(nc, a, b, c)])
-    const double corr = (27.0 * EH(I, J, K) + 9.0 * (EH(I2, J, K) + EH(I, J2, K) + EH(I, J, K2)) +
-                         3.0 * (EH(I2, J2, K) + EH(I2, J, K2) + EH(I, J2, K2)) + EH(I2, J2, K2)) *
-                        (1.0 / 64.0);
-#undef EH
-    const double old = uf[t];
-    double v = old + corr;
-    if (FR && !(v > 0.0)) {
-      v = 0.5 * old;
-      count_guards(guard, 1u);
+  const int Iv[3] = {wrapi(i - 1, nc), i, wrapi(i + 1, nc)};
+  const int Jv[3] = {wrapi(j - 1, nc), j, wrapi(j + 1, nc)};
+  const int Kv[3] = {wrapi(k - 1, nc), k, wrapi(k + 1, nc)};
+  double jk[3][2][2];  // [I offset][j child][k child]
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    double r[3][2];  // [J offset][k child]
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+      double d[3];
+#pragma unroll
+      for (int z = 0; z < 3; ++z) {
+        const size_t t = cidx(nc, Iv[x], Jv[y], Kv[z]);
+        d[z] = uH[t] - RuH[t];
+      }
+      r[y][0] = fma(3.0, d[1], d[0]);
+      r[y][1] = fma(3.0, d[1], d[2]);
     }
-    uf[t] = v;
+#pragma unroll
+    for (int ck = 0; ck < 2; ++ck) {
+      jk[x][0][ck] = fma(3.0, r[1][ck], r[0][ck]);
+      jk[x][1][ck] = fma(3.0, r[1][ck], r[2][ck]);
+    }
   }
+  unsigned ng = 0;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int ck = 0; ck < 2; ++ck) {
+        const double corr = fma(3.0, jk[1][b][ck], jk[a ? 2 : 0][b][ck]);
+        const size_t t = cidx(nf, 2 * i + a, 2 * j + b, 2 * k + ck);
+        const double old = uf[t];
+        double v = fma(corr, 1.0 / 64.0, old);
+        if (FR && !(v > 0.0)) {
+          v = 0.5 * old;
+          ++ng;
+        }
+        uf[t] = v;
+      }
+  if (FR) count_guards(guard, ng);
 }
 
-// Coarsest level: 'sweeps' red-black sweeps by one CTA (the level is tiny).
+// Coarsest level: 'sweeps' red-black sweeps by one CTA (the level is tiny), the
+// field in shared memory; a thread's cells are the same in every sweep.
+constexpr int kCoarseThreads = 512;
 template <int K>
-__global__ void __launch_bounds__(512) k_coarse64(ModelDev m, int n, double h, double* __restrict__ u,
-                                                  const double* __restrict__ rho,
-                                                  const double* __restrict__ S, int sweeps) {
-  const int n3 = n * n * n;
-  for (int s = 0; s < sweeps; ++s) {
-    for (int parity = 0; parity < 2; ++parity) {
-      for (int t = threadIdx.x; t < n3; t += blockDim.x) {
-        const int k = t % n, j = (t / n) % n, i = t / (n * n);
-        if (((i + j + k) & 1) != parity) continue;
-        const double Lnb = nb_sum64<K>(u, n, i, j, k);
-        u[t] = local_update64<K>(m, h, u[t], rho[t], S ? S[t] : 0.0, Lnb);
-      }
-      __syncthreads();
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse64(Const64 c, int n, double* __restrict__ u,
+                                                             const double* __restrict__ rho,
+                                                             const double* __restrict__ S, int sweeps) {
+  extern __shared__ double su[];
+  const int n3 = n * n * n, h = n >> 1;
+  for (int t = threadIdx.x; t < n3; t += blockDim.x) su[t] = u[t];
+  __syncthreads();
+  for (int s = 0; s < 2 * sweeps; ++s) {
+    // the s & 1 colour: cell kk of row (i, j), k = 2 kk + (i + j + s) & 1 (an odd row length
+    // leaves its last cell to the colour of even k)
+    for (int t = threadIdx.x; t < (h + (n & 1)) * n * n; t += blockDim.x) {
+      const int w = h + (n & 1), kk = t % w, r = t / w, j = r % n, i = r / n;
+      const int k = 2 * kk + ((i + j + s) & 1);
+      if (k >= n) continue;
+      const int o = (i * n + j) * n + k;
+      const double Lnb = nb_sum64<K>(su, n, i, j, k);
+      su[o] = local_update64<K>(c, su[o], rho[o], S ? S[o] : 0.0, Lnb);
     }
+    __syncthreads();
   }
+  for (int t = threadIdx.x; t < n3; t += blockDim.x) u[t] = su[t];
 }
 
 __global__ void k_sum_f32(const float* __restrict__ x, long long n3, double* __restrict__ partials) {
@@ -294,9 +290,9 @@ __global__ void k_init_background_first(double* __restrict__ field, double ubar)
 // Launchers (dispatch on the model kind)
 // ---------------------------------------------------------------------------
 
-// 3D grid for kernels indexed (x: k, y: j, z: i) with k3dThreads threads along k.
-constexpr int k3dThreads = 64;
-static dim3 grid3d(int n_k, int n_j, int n_i) { return dim3((n_k + k3dThreads - 1) / k3dThreads, n_j, n_i); }
+// Grid of the 3D kernels (x: k, y: j, z: i) for blocks of kTx x kTy threads.
+static dim3 grid3d(int n_k, int n_j, int n_i) { return dim3((n_k + kTx - 1) / kTx, (n_j + kTy - 1) / kTy, n_i); }
+static const dim3 kBlock3(kTx, kTy);
 
 #define MG_DISPATCH(kind, KERNEL_CALL)                       \
   switch (kind) {                                            \
@@ -311,9 +307,10 @@ static dim3 grid3d(int n_k, int n_j, int n_i) { return dim3((n_k + k3dThreads - 
 int launch_smooth64(const ModelDev& m, int n, double h, double* u, const double* rho, const double* S,
                     int sweeps, cudaStream_t st) {
   const dim3 g = grid3d(n / 2, n, n);
+  const Const64 c = make_const64(m, h);
   for (int s = 0; s < sweeps; ++s)
     for (int parity = 0; parity < 2; ++parity) {
-      MG_DISPATCH(m.kind, (k_smooth64<KK><<<g, k3dThreads, 0, st>>>(m, n, h, u, rho, S, parity)));
+      MG_DISPATCH(m.kind, (k_smooth64<KK><<<g, kBlock3, 0, st>>>(c, n, u, rho, S, parity)));
     }
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
@@ -324,7 +321,7 @@ int launch_residual64(const ModelDev& m, int n, double h, const double* u, const
   const long long n3 = (long long)n * n * n;
   const int g = n * n < 2048 ? n * n : 2048;
   const int bt = n >= 256 ? 256 : (n <= 32 ? 32 : ((n + 31) / 32) * 32);
-  MG_DISPATCH(m.kind, (k_residual64<KK><<<g, bt, 0, st>>>(m, n, h, u, rho, S, d, partials)));
+  MG_DISPATCH(m.kind, (k_residual64<KK><<<g, bt, 0, st>>>(make_const64(m, h), n, u, rho, S, d, partials)));
   k_finalize_sum<<<1, 1024, 0, st>>>(partials, g, out_sum);
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
@@ -332,8 +329,7 @@ int launch_residual64(const ModelDev& m, int n, double h, const double* u, const
 }
 
 int launch_restrict64(int nf, const double* fine, double* coarse, cudaStream_t st) {
-  const long long nc3 = (long long)(nf / 2) * (nf / 2) * (nf / 2);
-  k_restrict64<<<grid3d(nf / 2, nf / 2, nf / 2), k3dThreads, 0, st>>>(nf, fine, coarse);
+  k_restrict64<<<grid3d(nf / 2, nf / 2, nf / 2), kBlock3, 0, st>>>(nf, fine, coarse);
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
@@ -341,10 +337,9 @@ int launch_restrict64(int nf, const double* fine, double* coarse, cudaStream_t s
 
 int launch_prolong_correct64(const ModelDev& m, int nc, const double* uH, const double* RuH,
                              unsigned long long* guard, double* uf, cudaStream_t st) {
-  const long long nf3 = 8LL * nc * nc * nc;
-  const dim3 g = grid3d(2 * nc, 2 * nc, 2 * nc);
-  if (is_fr(m.kind)) k_prolong_correct64<true><<<g, k3dThreads, 0, st>>>(nc, uH, RuH, uf, guard);
-  else k_prolong_correct64<false><<<g, k3dThreads, 0, st>>>(nc, uH, RuH, uf, guard);
+  const dim3 g = grid3d(nc, nc, nc);
+  if (is_fr(m.kind)) k_prolong_correct64<true><<<g, kBlock3, 0, st>>>(nc, uH, RuH, uf, guard);
+  else k_prolong_correct64<false><<<g, kBlock3, 0, st>>>(nc, uH, RuH, uf, guard);
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
@@ -353,25 +348,34 @@ int launch_prolong_correct64(const ModelDev& m, int nc, const double* uH, const 
 int launch_coarse64(const ModelDev& m, int n, double h, double* u, const double* rho, const double* S,
                     int sweeps, cudaStream_t st) {
   if ((long long)n * n * n > 4096) return launch_smooth64(m, n, h, u, rho, S, sweeps, st);
-  MG_DISPATCH(m.kind, (k_coarse64<KK><<<1, 512, 0, st>>>(m, n, h, u, rho, S, sweeps)));
+  const size_t smem = (size_t)n * n * n * sizeof(double);  // at most 32 KB
+  MG_DISPATCH(m.kind, (k_coarse64<KK><<<1, kCoarseThreads, smem, st>>>(make_const64(m, h), n, u, rho, S, sweeps)));
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
 }
 
 int launch_residual_restrict64(const ModelDev& m, int nf, double hf, const double* u, const double* rho,
-                               const double* S, double* Ru, double* uH, double* Rd, cudaStream_t st) {
-  const long long nc3 = (long long)(nf / 2) * (nf / 2) * (nf / 2);
+                               const double* S, double* Ru, double* uH, double* Rd, bool relaxed, cudaStream_t st) {
   const dim3 g = grid3d(nf / 2, nf / 2, nf / 2);
-  MG_DISPATCH(m.kind, (k_residual_restrict64<KK><<<g, k3dThreads, 0, st>>>(m, nf, hf, u, rho, S, Ru, uH, Rd)));
+  const Const64 c = make_const64(m, hf);
+  if (relaxed && m.kind != KCQ) {
+    switch (m.kind) {
+      case KFR0: k_residual_restrict64<KFR0, true><<<g, kBlock3, 0, st>>>(c, nf, u, rho, S, Ru, uH, Rd); break;
+      case KFR1: k_residual_restrict64<KFR1, true><<<g, kBlock3, 0, st>>>(c, nf, u, rho, S, Ru, uH, Rd); break;
+      case KFR2: k_residual_restrict64<KFR2, true><<<g, kBlock3, 0, st>>>(c, nf, u, rho, S, Ru, uH, Rd); break;
+      default: k_residual_restrict64<KSYM, true><<<g, kBlock3, 0, st>>>(c, nf, u, rho, S, Ru, uH, Rd); break;
+    }
+    note_launch(1);
+  } else {
+    MG_DISPATCH(m.kind, (k_residual_restrict64<KK, false><<<g, kBlock3, 0, st>>>(c, nf, u, rho, S, Ru, uH, Rd)));
+  }
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
 }
 
 int launch_fas_source64(const ModelDev& m, int nc, double hc, const double* Ru, const double* rho, double* S,
                         cudaStream_t st) {
-  const long long n3 = (long long)nc * nc * nc;
-  const int g = grid_for(n3, kThreads, 1 << 20);
-  MG_DISPATCH(m.kind, (k_fas_source64<KK><<<grid3d(nc, nc, nc), k3dThreads, 0, st>>>(m, nc, hc, Ru, rho, S)));
+  MG_DISPATCH(m.kind, (k_fas_source64<KK><<<grid3d(nc, nc, nc), kBlock3, 0, st>>>(make_const64(m, hc), nc, Ru, rho, S)));
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
 }
@@ -427,7 +431,7 @@ static int vcycle64(const ModelDev& m, Workspace* ws, int l, const mgglam_params
   Level& C = ws->lev[l + 1];
   // Ru -> C.Ru, u^H = Ru -> C.u, R d -> C.S (then C.S <- N^H(Ru) - R d)
   if (l == 0) prof_begin(PC_RESTRICT64_FINE, st, (16.0 + 3.0) * L.n3);
-  if ((rc = launch_residual_restrict64(m, L.n, L.h, L.u, L.rho, L.S, C.Ru, C.u, C.S, st))) return rc;
+  if ((rc = launch_residual_restrict64(m, L.n, L.h, L.u, L.rho, L.S, C.Ru, C.u, C.S, prm->nu1 > 0, st))) return rc;
   if (l == 0) { prof_end(st); prof_begin(PC_COARSE_LEVELS, st, 0.0); }
   if ((rc = launch_fas_source64(m, C.n, C.h, C.Ru, C.rho, C.S, st))) return rc;
   if ((rc = vcycle64(m, ws, l + 1, prm, st, mode))) return rc;
