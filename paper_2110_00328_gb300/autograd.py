@@ -29,7 +29,8 @@ class ScalarSolve(torch.autograd.Function):
     def forward(ctx, rho, log_fR0, prm: binding.Params, a: float, tol: float):
         p = replace(prm, fR0_abs=float(math.exp(float(log_fR0))))
         N = rho.shape[0]
-        field = torch.full((N, N, N), float("nan"), dtype=torch.float64, device=rho.device)
+        field = torch.empty((N, N, N), dtype=torch.float64, device=rho.device)
+        field.view(-1)[:1].fill_(float("nan"))  # the mark of a start from the background
         binding.solve_scalar(p, a, rho.contiguous(), field, tol)
         ctx.save_for_backward(rho, field)
         ctx.p, ctx.a, ctx.tol = p, a, tol
