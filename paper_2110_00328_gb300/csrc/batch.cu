@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(256) kb_outer_residual(const BFine* __restrict
   if (active[f.solve]) {
     const int tiles = (f.n / 32) * (f.n / 8);
     if constexpr (K == KCQ) {
-      a = outer_residual_tile<K, 8, 32>(f.m, f.n, 64, f.u, f.src, f.ub, f.tau, b % tiles, b / tiles);
+      a = cq_residual_tile<false, 8, 32, false>(f.m, CqSeries{}, 0.0, f.n, 64, f.u, f.src, nullptr, f.ub, f.tau,
+                                                b % tiles, b / tiles);
     } else {
       const FFC c = *f.ffc;
       a = outer_residual_tile_ff<K, 8, 32, true>(c, f.n, 64, f.u, f.rho, f.ub, f.tau, b % tiles, b / tiles);
@@ -748,8 +749,7 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
     const long long n3 = (long long)v.N * v.N * v.N;
     if ((rc = launch_density_mean(rho[s], (size_t)n3, B->partials, B->rmean + s, st))) return rc;
     if (models[s].kind == KCQ) {
-      MG_BDISPATCH(models[s].kind, (k_src64<KK><<<stream_grid(n3), kThreads, 0, st>>>(
-                                       models[s], rho[s], n3, B->rmean + s, v.src64)));
+      k_src64<<<stream_grid(n3), kThreads, 0, st>>>(rho[s], n3, B->rmean + s, v.src64);
     } else {
       k_ff_consts<<<1, 32, 0, st>>>(models[s], n3, B->rmean + s, B->ffc + s);
     }

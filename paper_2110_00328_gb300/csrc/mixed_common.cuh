@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "ff.cuh"
+#include "fp64_fast.cuh"
 #include "mg_common.cuh"
 #include "sweep32.cuh"
 
@@ -28,6 +29,7 @@ static inline LevelF make_levelf(const ModelDev& m, double h) {
   } else if (m.kind == KSYM) {
     f.al = (float)(m.c2 * m.xi2_a2 / (h * h));
     f.msym = (float)m.msym;
+    f.imsym = (float)(1.0 / m.msym);
     f.rat3 = (float)m.rat3;
   } else {
     f.cq_src = (float)m.cq_src;
@@ -37,6 +39,12 @@ static inline LevelF make_levelf(const ModelDev& m, double h) {
     f.inv_c2 = (float)(1.0 / m.c2);
     f.beta = (float)m.beta;
     f.keep_exp = m.keep_exp;
+    const double e1 = -1.0 - m.alpha, d = 1.0 / (m.c2 * m.phibar);
+    f.cq_lin = (float)(m.cq_pot * m.pot0 * e1 * d);
+    f.cq_d = (float)d;
+    f.cq_r2 = (float)((e1 - 1.0) / 2.0);
+    f.cq_r3 = (float)((e1 - 1.0) * (e1 - 2.0) / 6.0);
+    f.cq_series = !m.keep_exp && m.alpha <= 2.0;
   }
   return f;
 }
@@ -50,6 +58,9 @@ __device__ __forceinline__ float local_M(const LevelF& f, float u, float e, floa
   } else if constexpr (K == KSYM) {
     return f.c2_h2 * (Lnb - 6.f * e) - f.msym * ((rho * f.rat3 - 1.f) * e + e * (3.f * u * u + 3.f * u * e + e * e));
   } else {
+    const float du = u * f.cq_d, dU = du + e * f.cq_d;
+    if (f.cq_series && fabsf(du) <= kCqSmall && fabsf(dU) <= kCqSmall)
+      return fmaf(Lnb - 6.f * e, f.ih2, cq_dpot(f, e, du, dU));
     const float x0 = f.phibar + u * f.inv_c2;
     const float dpow = powf(x0, -1.f - f.alpha) * expm1f((-1.f - f.alpha) * log1pf(e * f.inv_c2 / x0));
     float v = (Lnb - 6.f * e) * f.ih2 + f.cq_pot * dpow;
@@ -92,7 +103,8 @@ __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast
 // clamped quad and store nothing.
 // QH (f(R) n = 1, 2 on a split level with stored q, in qf): the halo rows'
 // neighbour quantities are read from qf instead of formed from e and u.
-// ZR (f(R), symmetron, after pre-smoothing): the second colour ((i+j+k) odd)
+// ZR (after pre-smoothing; f(R), symmetron, and CQ where its one Newton step solves
+// the cell's equation to rounding, cq_linear): the second colour ((i+j+k) odd)
 // was relaxed last and satisfies its local equations, so its defect is taken as
 // zero and only the first colour's is formed (see restrict_split_zr).
 template <int K, class FL = NatLayout, bool QH = false, bool ZR = false>
@@ -172,7 +184,6 @@ __device__ __forceinline__ void restrict_quad(const LevelF& f, int nf, const flo
       }
       const float4 Ev = E[a][b], Uv = U[a][b];
       // with ZR the cells k0 + c of colour (a + b + c) & 1 = 1 have zero defect (k0, 2I, 2J even)
-      static_assert(!ZR || K != KCQ, "CQ relaxes by one Newton step: its defect is not zero");
       const bool odd = (a + b) & 1;
       float dx = 0.f, dy = 0.f, dz = 0.f, dv = 0.f;
       if (!ZR || !odd) {
@@ -455,7 +466,9 @@ __device__ __forceinline__ void prolong_quad(int nc, const float* __restrict__ e
 // of the coarse row pair (I, J) -- which interpolate from the nine coarse rows
 // (I-1..I+1, J-1..J+1); prolong_quad reads four coarse rows for each fine row.
 // Each fine row's second-colour pair is corrected (and its q written) exactly
-// as prolong_quad<true, SplitLayout, QK, true> does it.  Grid as the
+// as prolong_quad<true, SplitLayout, QK, true> does it.  QK < 0: the models whose
+// neighbour quantity is e itself (symmetron; CQ where cq_linear), which need
+// neither the guard nor q.  Grid as the
 // restriction's: (ceil(nf/128), nc [J], ceil(nc/4) [I]), block (32, 4).
 // DD: eH holds the coarse difference eH - Re itself (written by the coarse
 // level's last post-smoothing pass, smooth_quad's WD), and Re is not read.
@@ -464,7 +477,7 @@ __device__ __forceinline__ void prolong_split2x2_second(int nc, const float* __r
                                                         const float* __restrict__ Re, const float* __restrict__ ub,
                                                         float* __restrict__ ef, int I, int J, int tq, int lane,
                                                         unsigned long long* guard, float* __restrict__ qf) {
-  static_assert(QK == KFR1 || QK == KFR2, "stored q: f(R) n = 1, 2");
+  static_assert(QK < 0 || QK == KFR1 || QK == KFR2, "stored q: f(R) n = 1, 2");
   const int nf = nc << 1, nq = nf >> 2, h = nf >> 1;
   const bool act = tq < nq;
   const int t = act ? tq : nq - 1;
@@ -512,53 +525,71 @@ __device__ __forceinline__ void prolong_split2x2_second(int nc, const float* __r
       const float cB = odd ? (3.f * Ry + Rx) * w : (3.f * Ry + Rp) * w;
       const int i = 2 * I + a, j = 2 * J + b;
       const IT o1 = H + ((IT)i * nf + j) * h + (k0 >> 1);
-      const float2 old = ld2(ef + o1), u = ld2(ub + o1);
+      const float2 old = ld2(ef + o1);
       float vA = old.x + cA, vB = old.y + cB;
-      const bool gA = !(u.x + vA > 0.f), gB = !(u.y + vB > 0.f);
-      if (gA) vA = 0.5f * (old.x - u.x);
-      if (gB) vB = 0.5f * (old.y - u.y);
-      ng += (unsigned)gA + (unsigned)gB;
-      if (act) {
-        *reinterpret_cast<float2*>(ef + o1) = make_float2(vA, vB);
-        *reinterpret_cast<float2*>(qf + o1) = make_float2(dw<QK>(u.x, vA), dw<QK>(u.y, vB));
+      if constexpr (QK >= 0) {
+        const float2 u = ld2(ub + o1);
+        const bool gA = !(u.x + vA > 0.f), gB = !(u.y + vB > 0.f);
+        if (gA) vA = 0.5f * (old.x - u.x);
+        if (gB) vB = 0.5f * (old.y - u.y);
+        ng += (unsigned)gA + (unsigned)gB;
+        if (act) *reinterpret_cast<float2*>(qf + o1) = make_float2(dw<QK>(u.x, vA), dw<QK>(u.y, vB));
       }
+      if (act) *reinterpret_cast<float2*>(ef + o1) = make_float2(vA, vB);
     }
-  if (act) count_guards(guard, ng);
+  if (QK >= 0 && act) count_guards(guard, ng);
 }
 
-// 1/x in FP64 by one Newton-Raphson refinement y1 = y0 (2 - x y0) of a
-// single-precision reciprocal y0: the relative error of y0 (below 2^-22) is
-// squared, leaving about 2^-44 ~ 6e-14, far below what the residual needs.
-__device__ __forceinline__ double rcp_nr(double x, float xf) {
-  const double y = (double)__frcp_rn(xf);
-  const double t = fma(-x, y, 1.0);
-  return fma(y, t, y);
-}
+// Whether one Newton step of CQ solves a cell's equation of this level to FP32
+// rounding: what it leaves, (cq_lin h^2 / 6) r2 d of the step, is below 4e-7.
+static inline bool cq_linear(const LevelF& f) { return f.cq_series && fabsf(f.cq_lin) <= 0x1p-10f * f.ih2; }
 
-// src64 = the part of N that does not depend on u, in FP64:
-// f(R): Om (rho/mean - 1)/a + Rbar a^2/3; symmetron: rho/mean (the density
-// itself, used in the u-dependent term); CQ: -3 beta Om e^{beta phibar}/a (rho/mean - 1).
-template <int K>
-__global__ void k_src64(ModelDev m, const float* __restrict__ rho32, long long n3, const double* __restrict__ rho_sum,
-                        double* __restrict__ src) {
+// CQ: the normalised density rho/mean in FP64 (the general residual's).
+static __global__ void k_src64(const float* __restrict__ rho32, long long n3, const double* __restrict__ rho_sum,
+                               double* __restrict__ src) {
   const double inv_mean = (double)n3 / *rho_sum;
-  // f(R): Om/a (rho/mean - 1) + K0 = c1 rho + c0, one FMA per cell
-  const double c1 = is_fr(K) ? m.om_a * inv_mean : inv_mean;
-  const double c0 = is_fr(K) ? m.K0 - m.om_a : 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x)
-    src[t] = fma(c1, (double)rho32[t], c0);
+    src[t] = inv_mean * (double)rho32[t];
 }
 
-// r = N(u64) on the fine level, z-marching tiles (each cell's transformed value
-// formed once): writes ub = float(u64), tau = float(-r), and per-block partial
-// sums of r^2 (accumulated from the float tau).
+// CQ's FP64 residual with the potential by its series (CqSeries::ok): the linear term
+// in FP64, the rest of the series in FP32.  The rest is at most 2^-10 of the linear
+// term (kCqSmall) and that at most 2^-18 of the field, so its rounding, 2^-52 of
+// the field, is FP64's own.
+struct CqSeries {
+  double lin;          // cq_pot pot0 (-1-alpha) / (c~^2 phibar)
+  float lf, d, r2, r3, r4;
+  int ok;
+};
+
+static inline CqSeries make_cq_series(const ModelDev& m) {
+  CqSeries c = {};
+  if (m.kind != KCQ) return c;
+  const double e1 = -1.0 - m.alpha, d = 1.0 / (m.c2 * m.phibar);
+  c.lin = m.cq_pot * m.pot0 * e1 * d;
+  c.lf = (float)c.lin;
+  c.d = (float)d;
+  c.r2 = (float)((e1 - 1.0) / 2.0);
+  c.r3 = (float)((e1 - 1.0) * (e1 - 2.0) / 6.0);
+  c.r4 = (float)((e1 - 1.0) * (e1 - 2.0) * (e1 - 3.0) / 24.0);
+  c.ok = !m.keep_exp && m.alpha <= 2.0 && fabs(c.lin) <= 0x1p-18;
+  return c;
+}
+
+// CQ's r = N(u64) on the fine level, z-marching tiles: writes ub = float(u64), tau =
+// float(-r), in the red-black split layout if SPLIT, and per-block partial sums of
+// r^2 (accumulated from the float tau).
 // Body for one CTA: tile index 'tile' over (j,k) tiles, chunk index 'cb' along i;
 // returns the CTA's sum of tau^2 (valid in thread 0).
-template <int K, int TJ, int TK>
-__device__ __forceinline__ double outer_residual_tile(const ModelDev& m, int n, int chunk, const double* __restrict__ u,
-                                                      const double* __restrict__ src, float* __restrict__ ub,
-                                                      float* __restrict__ tau, int tile, int cb) {
+// SERIES: the potential by its series, the source from the caller's density (cq1 =
+// -cq_src / mean): ten FP64 instructions a cell, which bound it; with pow, ~150.
+// Measured at 128^3: 58 us against 490 us.
+template <bool SERIES, int TJ, int TK, bool SPLIT>
+__device__ __forceinline__ double cq_residual_tile(const ModelDev& m, const CqSeries& q, double cq1, int n, int chunk,
+                                                   const double* __restrict__ u, const double* __restrict__ src,
+                                                   const float* __restrict__ rho, float* __restrict__ ub,
+                                                   float* __restrict__ tau, int tile, int cb) {
   constexpr int PJ = TJ + 2, PK = TK + 2, PS = PJ * PK;
   __shared__ double s_w[3][PS];
   const int tiles_k = n / TK;
@@ -577,8 +608,7 @@ __device__ __forceinline__ double outer_residual_tile(const ModelDev& m, int n, 
     const size_t base = (size_t)ig * n * n;
     for (int c = t; c < PS; c += TJ * TK) {
       const int jj = c / PK, kk = c - jj * PK;
-      const size_t g = base + (size_t)wrapi(j0 + jj - 1, n) * n + wrapi(k0 + kk - 1, n);
-      s_w[slot][c] = fr_or_id<K>(u[g]);
+      s_w[slot][c] = u[base + (size_t)wrapi(j0 + jj - 1, n) * n + wrapi(k0 + kk - 1, n)];
     }
   };
   load(i0 - 1);
@@ -588,23 +618,30 @@ __device__ __forceinline__ double outer_residual_tile(const ModelDev& m, int n, 
     __syncthreads();
     const int sl = (i + 3) % 3, sm = (i + 2) % 3, sp = (i + 4) % 3;
     const size_t g = ((size_t)i * n + jg) * n + kg;
-    const double uc = u[g];
+    const double uc = s_w[sl][cc];
     const double L = s_w[sm][cc] + s_w[sp][cc] + s_w[sl][cc - PK] + s_w[sl][cc + PK] + s_w[sl][cc - 1] +
                      s_w[sl][cc + 1];
-    const float uf = (float)uc;
+    const float uf = SERIES ? d2f_bits(uc) : (float)uc;
     double v;
-    if constexpr (is_fr(K)) {
-      v = fma(-m.c2, L - 6.0 * s_w[sl][cc], src[g]) - m.K * rcp_nr(uc, uf);
-    } else if constexpr (K == KSYM) {
-      v = m.c2 * (L - 6.0 * uc) - m.msym * ((src[g] * m.rat3 - 1.0) * uc + uc * uc * uc);
+    if constexpr (SERIES) {
+      const double lap = fma(-6.0, uc, L);
+      const double sc = fma(cq1, f2d_bits(rho[g]), m.cq_src);
+      const float d = uf * q.d;
+      if (fabsf(d) <= kCqSmall) {
+        const float rest = q.lf * uf * d * fmaf(d, fmaf(d, q.r4, q.r3), q.r2);
+        v = lap + fma(q.lin, uc, sc + f2d_bits(rest));
+      } else {
+        v = lap + sc + m.cq_pot * (pow(m.phibar + uc / m.c2, -1.0 - m.alpha) - m.pot0);
+      }
     } else {
       const double E = m.keep_exp ? exp(m.beta * uc / m.c2) : 1.0;
       const double x = m.phibar + uc / m.c2;
       v = (L - 6.0 * uc) - m.cq_src * (E * src[g] - 1.0) + m.cq_pot * (pow(x, -1.0 - m.alpha) - m.pot0);
     }
-    const float tv = (float)(-v);
-    ub[g] = uf;
-    tau[g] = tv;
+    const float tv = SERIES ? -d2f_bits(v) : (float)(-v);
+    const size_t o = SPLIT ? (size_t)split_idx(n, i, jg, kg) : g;
+    ub[o] = uf;
+    tau[o] = tv;
     acc += tv * tv;
     __syncthreads();
   }
@@ -622,6 +659,7 @@ struct FFC {
   ff K;       // f(R): K0 ubar
   ff c1, c0;  // source term c1 rho + c0: f(R) Om/(a mean), K0 - Om/a; symmetron 1/mean, 0
   ff msym, rat3;
+  double cq1;  // CQ: -cq_src / mean
 };
 
 __device__ __forceinline__ ff ff_split_dev(double d) {
@@ -641,6 +679,7 @@ static __global__ void k_ff_consts(ModelDev m, long long n3, const double* __res
   c.c0 = ff_split_dev(fr ? m.K0 - m.om_a : 0.0);
   c.msym = ff_split_dev(m.msym);
   c.rat3 = ff_split_dev(m.rat3);
+  c.cq1 = -m.cq_src * inv_mean;
   *out = c;
 }
 
@@ -1084,14 +1123,16 @@ static __global__ void k_background_first(const double* __restrict__ u, int* __r
   *flag = isnan(u[0]) ? 1 : 0;
 }
 
-template <int K, int TJ, int TK>
-__global__ void __launch_bounds__(TJ* TK) k_outer_residual(ModelDev m, int n, int chunk, const double* __restrict__ u,
-                                                           const double* __restrict__ src, float* __restrict__ ub,
-                                                           float* __restrict__ tau, double* __restrict__ partials) {
-  const double a = outer_residual_tile<K, TJ, TK>(m, n, chunk, u, src, ub, tau, blockIdx.x, blockIdx.y);
+template <bool SERIES, int TJ, int TK, bool SPLIT>
+__global__ void __launch_bounds__(TJ* TK) k_cq_residual(ModelDev m, CqSeries q, const FFC* __restrict__ C, int n,
+                                                        int chunk, const double* __restrict__ u,
+                                                        const double* __restrict__ src, const float* __restrict__ rho,
+                                                        float* __restrict__ ub, float* __restrict__ tau,
+                                                        double* __restrict__ partials) {
+  const double a = cq_residual_tile<SERIES, TJ, TK, SPLIT>(m, q, SERIES ? C->cq1 : 0.0, n, chunk, u, src, rho, ub, tau,
+                                                           blockIdx.x, blockIdx.y);
   if (threadIdx.x == 0) partials[blockIdx.x + blockIdx.y * gridDim.x] = a;
 }
-
 
 // ---- small whole-mesh kernels shared by the single and batched solvers ----
 

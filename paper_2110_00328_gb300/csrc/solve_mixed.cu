@@ -324,6 +324,7 @@ struct MixedCtx {
   const float* rho;   // the caller's density (the float-float residual forms its source from it)
   bool split;         // the finest level in the red-black split layout
   bool ff_resid;      // fine residual in float-float (f(R), symmetron) rather than FP64 (CQ)
+  CqSeries cq;        // CQ: the potential's series
   int tail_level;     // first level (>= 1) run by the one-block tail kernel, or -1
   float* qs;          // split f(R) n = 1, 2: the finest level's stored neighbour quantity, else nullptr
   unsigned long long* guard;  // positivity-guard replacements of this solve (workspace scalar)
@@ -484,18 +485,18 @@ static int smooth32(const MixedCtx& C, int l, int sweeps, cudaStream_t st, bool 
         if (np <= 0) return MGGLAM_OK;
         if (split) {
           const unsigned blocks = (unsigned)((split_warps(L.n, np) + 3) / 4);
+          // programmatic dependent launch: a pass overlaps its start with the
+          // previous pass's last wave (the first pass of the call waits first)
+          cudaLaunchConfig_t cfg = {};
+          cfg.gridDim = dim3(blocks);
+          cfg.blockDim = dim3(32, 4);
+          cfg.stream = st;
+          cudaLaunchAttribute attr[2];
+          attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+          attr[0].val.programmaticStreamSerializationAllowed = 1;
+          cfg.attrs = attr;
+          cfg.numAttrs = 1;
           if (C.qs) {
-            // programmatic dependent launch: a pass overlaps its start with the
-            // previous pass's last wave (the first pass of the call waits first)
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(blocks);
-            cfg.blockDim = dim3(32, 4);
-            cfg.stream = st;
-            cudaLaunchAttribute attr[2];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
             if (C.l2 && C.l2->ok) {
               attr[1].id = cudaLaunchAttributeAccessPolicyWindow;
               attr[1].val.accessPolicyWindow = C.l2->w;
@@ -522,8 +523,13 @@ static int smooth32(const MixedCtx& C, int l, int sweeps, cudaStream_t st, bool 
             note_launch(1);
             return MGGLAM_OK;
           }
-          MG_DISPATCH32(C.m.kind, (k_smooth32s<KK><<<blocks, dim3(32, 4), 0, st>>>(C.lf[l], L.n, L.e, L.ub, rho,
-                                                                                   L.S32, parity, i0, np, nullptr, 0)));
+          const int pdl = passes++ > 0 ? 1 : 2;
+          auto go = [&](auto kern) {
+            return cudaLaunchKernelEx(&cfg, kern, C.lf[l], L.n, L.e, (const float*)L.ub, rho, (const float*)L.S32,
+                                      parity, i0, np, (float*)nullptr, pdl);
+          };
+          const bool i32 = L.n <= 1024;
+          MG_DISPATCH32(C.m.kind, MG_CUDA_TRY(i32 ? go(k_smooth32s<KK, false, 0, int>) : go(k_smooth32s<KK>)));
           return MGGLAM_OK;
         }
         const dim3 g((L.n / 4 + 31) / 32, L.n, (np + 3) / 4);
@@ -567,14 +573,22 @@ static int smooth32(const MixedCtx& C, int l, int sweeps, cudaStream_t st, bool 
 
 static int vcycle32(const MixedCtx& C, int l, cudaStream_t st, int mode);
 
+// Whether the first pass after the finest level's prolongation takes nothing from
+// the first colour's old values (to rounding), so that only the second colour has
+// to be corrected when post-smoothing follows: a split level, f(R) n = 1, 2 (with
+// the stored q), the symmetron, and CQ where one Newton step solves a cell.
+static bool second_colour_only(const MixedCtx& C) {
+  return C.split && (C.qs || C.m.kind == KSYM || (C.m.kind == KCQ && cq_linear(C.lf[0])));
+}
+
 // Whether the finest level's second-colour prolongation reads the coarse
 // difference eH - Re that level 1's last post-smoothing sweep stores in its
 // second buffer (unused there: the split layout excludes the fused sweep): a
-// split f(R) n = 1, 2 finest level with post-smoothing, whose level 1 is smoothed
+// split finest level so prolonged, with post-smoothing, whose level 1 is smoothed
 // by the quad kernel (neither the coarsest, a tail, nor slab-scheduled).
 static bool fine_reads_d(const MixedCtx& C) {
   const Workspace* ws = C.ws;
-  if (!(C.split && C.qs && C.prm->nu2 >= 1 && ws->nlev > 2 && C.tail_level != 1)) return false;
+  if (!(second_colour_only(C) && C.prm->nu2 >= 1 && ws->nlev > 2 && C.tail_level != 1)) return false;
   const int n1 = ws->lev[1].n;
   return n1 % 4 == 0 && n1 >= 16 && !use_fused(C, n1) && slab_planes(C, n1) == 0 && ws->lev[1].e_alt;
 }
@@ -714,9 +728,9 @@ static void tail_allow_smem() {
   cudaFuncSetAttribute(k_tail32<KCQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-// The natural-layout restriction after pre-smoothing (ZR), per model kind.
+// The restriction after pre-smoothing (ZR) of a level in layout FL, per model kind.
 template <class FL, bool ZR>
-static void launch_restrict_nat(const MixedCtx& C, int l, const float* rho, dim3 g, cudaStream_t st) {
+static void launch_restrict_quad(const MixedCtx& C, int l, const float* rho, dim3 g, cudaStream_t st) {
   Level& L = C.ws->lev[l];
   Level& H = C.ws->lev[l + 1];
   switch (C.m.kind) {
@@ -726,7 +740,9 @@ static void launch_restrict_nat(const MixedCtx& C, int l, const float* rho, dim3
                    C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr); break;
     case KFR2: k_residual_restrict32q<KFR2, FL, false, ZR><<<g, dim3(32, 4), 0, st>>>(
                    C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr); break;
-    default: k_residual_restrict32q<KSYM, FL, false, ZR><<<g, dim3(32, 4), 0, st>>>(
+    case KSYM: k_residual_restrict32q<KSYM, FL, false, ZR><<<g, dim3(32, 4), 0, st>>>(
+                   C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr); break;
+    default: k_residual_restrict32q<KCQ, FL, false, ZR><<<g, dim3(32, 4), 0, st>>>(
                    C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr); break;
   }
 }
@@ -758,6 +774,10 @@ static int restrict_level(const MixedCtx& C, int l, cudaStream_t st, bool relaxe
       k_residual_restrict32q<KFR2, SplitLayout, true><<<g, dim3(32, 4), 0, st>>>(C.lf[l], L.n, L.e, L.ub, rho, L.S32,
                                                                                  H.Re, H.e, H.ub, H.S32, C.qs);
       note_launch(1);
+    } else if (relaxed && (C.m.kind != KCQ || cq_linear(C.lf[l]))) {
+      if (L.n <= 1024) launch_restrict_quad<SplitLayout32, true>(C, l, rho, g, st);
+      else launch_restrict_quad<SplitLayout, true>(C, l, rho, g, st);
+      note_launch(1);
     } else {
       MG_DISPATCH32(C.m.kind, (k_residual_restrict32q<KK, SplitLayout><<<g, dim3(32, 4), 0, st>>>(
                                    C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr)));
@@ -765,9 +785,9 @@ static int restrict_level(const MixedCtx& C, int l, cudaStream_t st, bool relaxe
   } else if (L.n % 4 == 0 && L.n >= 8) {
     const dim3 g((L.n / 4 + 31) / 32, H.n, (H.n + 3) / 4);
     // 32-bit cell offsets where n^3 < 2^31
-    if (relaxed && C.m.kind != KCQ) {
-      if (L.n <= 1024) launch_restrict_nat<NatLayout32, true>(C, l, rho, g, st);
-      else launch_restrict_nat<NatLayout, true>(C, l, rho, g, st);
+    if (relaxed && (C.m.kind != KCQ || cq_linear(C.lf[l]))) {
+      if (L.n <= 1024) launch_restrict_quad<NatLayout32, true>(C, l, rho, g, st);
+      else launch_restrict_quad<NatLayout, true>(C, l, rho, g, st);
       note_launch(1);
     } else {
       if (L.n <= 1024) {
@@ -795,7 +815,7 @@ static int prolong_level(const MixedCtx& C, int l, cudaStream_t st, bool both = 
   if (l == 0 && C.split) {
     const dim3 g((L.n / 4 + 31) / 32, L.n, L.n / 4);
     // with post-smoothing the first colour's corrections would be overwritten unread (prolong_quad)
-    const bool second_only = !both && C.prm->nu2 >= 1;
+    const bool second_only = !both && C.prm->nu2 >= 1 && second_colour_only(C);
     const dim3 g2((L.n / 4 + 31) / 32, H.n, (H.n + 3) / 4);
     const bool dd = second_only && fine_reads_d(C);  // H.e_alt holds eH - Re
     const bool i32 = L.n <= 1024;  // 32-bit cell offsets
@@ -805,6 +825,12 @@ static int prolong_level(const MixedCtx& C, int l, cudaStream_t st, bool both = 
     else if (C.qs && C.m.kind == KFR2 && dd)
       (i32 ? k_prolong32_split2x2<KFR2, true, int> : k_prolong32_split2x2<KFR2, true>)<<<g2, dim3(32, 4), 0, st>>>(
           H.n, H.e_alt, H.Re, L.ub, L.e, C.guard, C.qs);
+    else if (!C.qs && second_only && dd)
+      (i32 ? k_prolong32_split2x2<-1, true, int> : k_prolong32_split2x2<-1, true>)<<<g2, dim3(32, 4), 0, st>>>(
+          H.n, H.e_alt, H.Re, L.ub, L.e, C.guard, nullptr);
+    else if (!C.qs && second_only)
+      (i32 ? k_prolong32_split2x2<-1, false, int> : k_prolong32_split2x2<-1>)<<<g2, dim3(32, 4), 0, st>>>(
+          H.n, H.e, H.Re, L.ub, L.e, C.guard, nullptr);
     else if (C.qs && C.m.kind == KFR1 && second_only)
       k_prolong32_split2x2<KFR1><<<g2, dim3(32, 4), 0, st>>>(H.n, H.e, H.Re, L.ub, L.e, C.guard, C.qs);
     else if (C.qs && C.m.kind == KFR2 && second_only)
@@ -867,7 +893,7 @@ static int vcycle32(const MixedCtx& C, int l, cudaStream_t st, int mode) {
   }
   // algorithmic bytes per fine cell: e, u read and e written (12), the coarse pair (1); the
   // second-colour-only form reads and writes half of e and u and writes half of q (9)
-  if (l == 0) { prof_end(st); prof_begin(PC_PROLONG32_FINE, st, (C.qs && C.prm->nu2 >= 1 ? 9.0 : 13.0) * L.n3); }
+  if (l == 0) { prof_end(st); prof_begin(PC_PROLONG32_FINE, st, (second_colour_only(C) && C.prm->nu2 >= 1 ? (C.qs ? 9.0 : 5.0) : 13.0) * L.n3); }
   if ((rc = prolong_level(C, l, st))) return rc;
   if (l == 0) { prof_end(st); prof_begin(PC_SMOOTH32_FINE, st, 16.0 * L.n3 * C.prm->nu2); }
   rc = smooth32(C, l, C.prm->nu2, st, l == 1 && fine_reads_d(C));
@@ -968,49 +994,55 @@ static int launch_outer_residual_ff(const MixedCtx& C, double* field, int* block
                                                                        ws->partials, skip);
     return MGGLAM_OK;
   }
-  const int tk = (F.n % 16 == 0) ? 16 : ((F.n % 8 == 0) ? 8 : ((F.n % 4 == 0) ? 4 : 2));
-  dim3 grid((F.n / tk) * (F.n / 2), 1);
-  *blocks = grid.x;
-  if (*blocks > kMaxReduceBlocks) return MGGLAM_ERR_SHAPE;
-  switch (tk) {
-    case 16: k_outer_residual_ff<K, 2, 16><<<grid, 32, 0, st>>>(ffc, F.n, F.n, field, C.rho, F.ub, F.S32, ws->partials); break;
-    case 8: k_outer_residual_ff<K, 2, 8><<<grid, 16, 0, st>>>(ffc, F.n, F.n, field, C.rho, F.ub, F.S32, ws->partials); break;
-    case 4: k_outer_residual_ff<K, 2, 4><<<grid, 8, 0, st>>>(ffc, F.n, F.n, field, C.rho, F.ub, F.S32, ws->partials); break;
-    default: k_outer_residual_ff<K, 2, 2><<<grid, 4, 0, st>>>(ffc, F.n, F.n, field, C.rho, F.ub, F.S32, ws->partials); break;
+  // small or non-tiling meshes: two rows of the widest dividing k-tile per CTA, its planes
+  // in chunks that fill the GPU
+  auto go = [&](auto kern, int tk) -> int {
+    const long long tiles = (long long)(F.n / tk) * (F.n / 2);
+    const int chunk = march_chunk(F.n, tiles, (const void*)kern, 2 * tk);
+    dim3 grid((unsigned)tiles, (F.n + chunk - 1) / chunk);
+    *blocks = grid.x * grid.y;
+    if (*blocks > kMaxReduceBlocks) return MGGLAM_ERR_SHAPE;
+    kern<<<grid, 2 * tk, 0, st>>>(ffc, F.n, chunk, field, C.rho, F.ub, F.S32, ws->partials, nullptr, nullptr, nullptr);
+    return MGGLAM_OK;
+  };
+  if (F.n % 16 == 0) return go(k_outer_residual_ff<K, 2, 16>, 16);
+  if (F.n % 8 == 0) return go(k_outer_residual_ff<K, 2, 8>, 8);
+  if (F.n % 4 == 0) return go(k_outer_residual_ff<K, 2, 4>, 4);
+  return go(k_outer_residual_ff<K, 2, 2>, 2);
+}
+
+// CQ's residual: FP64, tiled, with the potential's series where it holds.
+static int launch_cq_residual(const MixedCtx& C, double* field, int* blocks, cudaStream_t st) {
+  Workspace* ws = C.ws;
+  Level& F = ws->lev[0];
+  auto go = [&](auto kern, int tj, int tk) -> int {
+    const long long tiles = (long long)(F.n / tk) * (F.n / tj);
+    const int chunk = march_chunk(F.n, tiles, (const void*)kern, tj * tk);
+    dim3 grid((unsigned)tiles, (F.n + chunk - 1) / chunk);
+    *blocks = grid.x * grid.y;
+    if (*blocks > kMaxReduceBlocks) return MGGLAM_ERR_SHAPE;
+    kern<<<grid, tj * tk, 0, st>>>(C.m, C.cq, ffc_of(ws), F.n, chunk, field, ws->src64, C.rho, F.ub, F.S32, ws->partials);
+    return MGGLAM_OK;
+  };
+  const bool q = C.cq.ok;
+  if (bg_residual_tiled(F.n)) {
+    if (C.split) return q ? go(k_cq_residual<true, kRTJ, kRTK, true>, kRTJ, kRTK)
+                          : go(k_cq_residual<false, kRTJ, kRTK, true>, kRTJ, kRTK);
+    return q ? go(k_cq_residual<true, kRTJ, kRTK, false>, kRTJ, kRTK)
+             : go(k_cq_residual<false, kRTJ, kRTK, false>, kRTJ, kRTK);
   }
-  return MGGLAM_OK;
+  // small or non-tiling meshes: two rows of the widest dividing k-tile per CTA
+  if (F.n % 16 == 0) return q ? go(k_cq_residual<true, 2, 16, false>, 2, 16) : go(k_cq_residual<false, 2, 16, false>, 2, 16);
+  if (F.n % 8 == 0) return q ? go(k_cq_residual<true, 2, 8, false>, 2, 8) : go(k_cq_residual<false, 2, 8, false>, 2, 8);
+  if (F.n % 4 == 0) return q ? go(k_cq_residual<true, 2, 4, false>, 2, 4) : go(k_cq_residual<false, 2, 4, false>, 2, 4);
+  return q ? go(k_cq_residual<true, 2, 2, false>, 2, 2) : go(k_cq_residual<false, 2, 2, false>, 2, 2);
 }
 
 template <int K>
 static int launch_outer_residual_t(const MixedCtx& C, double* field, int* blocks, cudaStream_t st, bool bg_first,
                                    bool zero) {
-  Workspace* ws = C.ws;
-  Level& F = ws->lev[0];
-  if constexpr (K != KCQ) {
-    if (C.ff_resid) return launch_outer_residual_ff<K>(C, field, blocks, st, bg_first, zero);
-  }
-  if (F.n % kRTK == 0 && F.n % kRTJ == 0) {
-    const int chunk = march_chunk(F.n, (long long)(F.n / kRTK) * (F.n / kRTJ),
-                                  (const void*)k_outer_residual<K, kRTJ, kRTK>, kRTJ * kRTK);
-    dim3 grid((F.n / kRTK) * (F.n / kRTJ), (F.n + chunk - 1) / chunk);
-    *blocks = grid.x * grid.y;
-    if (*blocks > kMaxReduceBlocks) return MGGLAM_ERR_SHAPE;
-    k_outer_residual<K, kRTJ, kRTK><<<grid, kRTJ * kRTK, 0, st>>>(C.m, F.n, chunk, field, ws->src64, F.ub, F.S32,
-                                                                  ws->partials);
-  } else {
-    // small or non-tiling meshes: two rows of the widest dividing k-tile per CTA
-    const int tk = (F.n % 16 == 0) ? 16 : ((F.n % 8 == 0) ? 8 : ((F.n % 4 == 0) ? 4 : 2));
-    dim3 grid((F.n / tk) * (F.n / 2), 1);
-    *blocks = grid.x;
-    if (*blocks > kMaxReduceBlocks) return MGGLAM_ERR_SHAPE;
-    switch (tk) {
-      case 16: k_outer_residual<K, 2, 16><<<grid, 32, 0, st>>>(C.m, F.n, F.n, field, ws->src64, F.ub, F.S32, ws->partials); break;
-      case 8: k_outer_residual<K, 2, 8><<<grid, 16, 0, st>>>(C.m, F.n, F.n, field, ws->src64, F.ub, F.S32, ws->partials); break;
-      case 4: k_outer_residual<K, 2, 4><<<grid, 8, 0, st>>>(C.m, F.n, F.n, field, ws->src64, F.ub, F.S32, ws->partials); break;
-      default: k_outer_residual<K, 2, 2><<<grid, 4, 0, st>>>(C.m, F.n, F.n, field, ws->src64, F.ub, F.S32, ws->partials); break;
-    }
-  }
-  return MGGLAM_OK;
+  if constexpr (K == KCQ) return launch_cq_residual(C, field, blocks, st);
+  else return launch_outer_residual_ff<K>(C, field, blocks, st, bg_first, zero);
 }
 
 // Whether the outer residual pass can zero the finest level's e and q when the
@@ -1053,8 +1085,9 @@ int solve_mixed(const mgglam_params* prm, double a, const float* rho, int N, dou
   C.chunk = prm->sweep_chunk > 0 ? prm->sweep_chunk : 16;  // < 0: per-colour kernels only
   C.rho = rho;
   C.ff_resid = C.m.kind != KCQ;
-  // red-black split fine level: float-float residual with its 8 x 32 tiles, per-colour smoothing
-  C.split = C.ff_resid && prm->sweep_chunk <= 0 && C.ws->lev[0].n % 32 == 0;
+  C.cq = make_cq_series(C.m);
+  // red-black split fine level: residuals with 8 x 32 tiles, per-colour smoothing
+  C.split = prm->sweep_chunk <= 0 && C.ws->lev[0].n % 32 == 0;
   // the split level never runs the fused sweep, so its second buffer holds q
   C.qs = C.split && (C.m.kind == KFR1 || C.m.kind == KFR2) ? C.ws->lev[0].e_alt : nullptr;
   C.guard = guard_of(C.ws);
@@ -1075,13 +1108,9 @@ int solve_mixed(const mgglam_params* prm, double a, const float* rho, int N, dou
   const int g = stream_grid(n3);
   // FP64 density mean and source term; FP32 normalised pyramid where the inner operator needs it
   if ((rc = launch_density_mean(rho, F.n3, ws->partials, ws->scalars + SC_MEAN, st))) return rc;
-  if (C.ff_resid) {
-    k_ff_consts<<<1, 32, 0, st>>>(C.m, n3, ws->scalars + SC_MEAN, ffc_of(ws));
-    note_launch(1);
-  } else {
-    MG_DISPATCH32(C.m.kind, (k_src64<KK><<<stream_grid(n3), kThreads, 0, st>>>(
-                                 C.m, rho, n3, ws->scalars + SC_MEAN, ws->src64)));
-  }
+  if (C.ff_resid || C.cq.ok) k_ff_consts<<<1, 32, 0, st>>>(C.m, n3, ws->scalars + SC_MEAN, ffc_of(ws));
+  else k_src64<<<stream_grid(n3), kThreads, 0, st>>>(rho, n3, ws->scalars + SC_MEAN, ws->src64);
+  note_launch(1);
   if (C.need_rho) {
     if (C.split) k_density_norm32_split<<<stream_grid(n3), kThreads, 0, st>>>(rho, F.n, ws->scalars + SC_MEAN, F.rho32);
     else k_density_norm32<<<stream_grid(n3), kThreads, 0, st>>>(rho, n3, ws->scalars + SC_MEAN, F.rho32);

@@ -76,10 +76,8 @@ __device__ __forceinline__ void tail_smooth(const LevelF& f, int n, float* e, co
         const int k = 2 * kk + ((i + j + parity) & 1);
         const int c = (i * n + j) * n + k;
         const float Lnb = tail_nb_sum<K>(e, ub, n, i, j, k);
-        if constexpr (K == KFR1 || K == KFR2)
-          e[c] = update_e_warm<K>(f, ub[c], e[c], S[c], Lnb, __activemask());  // the lanes still in the loop
-        else
-          e[c] = update_e_fast<K>(f, ub[c], e[c], rho ? rho[c] : 1.f, S[c], Lnb);
+        // the lanes still in the loop together
+        e[c] = update_quad<K>(f, ub[c], e[c], rho ? rho[c] : 1.f, S[c], Lnb, __activemask());
       }
       __syncthreads();
     }
