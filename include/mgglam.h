@@ -93,7 +93,7 @@ typedef struct {
   int tail_cells;     /* MIXED: the coarsest levels, from the first level (below the finest)
                          with at most this many cells, run as one thread block with the
                          levels in shared memory (same arithmetic, fewer launches).
-                         0 (default) = 512; < 0 = off; at most 4096 */
+                         0 (default) = 4096, the most; < 0 = off */
   int cycle;          /* multigrid cycle: 0 (default) V, 1 F, 2 W (Sec. 3.2.1; each level
                          recurses once (V), twice (W), or F then V (F)) */
   int fmg;            /* 1: full-multigrid start (f(R), symmetron): the first cycle solves

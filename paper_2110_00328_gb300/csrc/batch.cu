@@ -3,9 +3,9 @@
 // All solves of a batch follow the mixed-precision scheme of solve_mixed.cu
 // (FP64 outer residual and update, FP32 correction-form FAS V-cycles) in lock
 // step.  Each phase of a V-cycle (one colour of smoothing on level l,
-// restriction l -> l+1, coarse source on l+1, coarsest-level relaxation,
-// prolongation l+1 -> l) is one kernel launch covering the blocks of every
-// solve that takes part in it: a block finds its solve by binary search in a
+// restriction l -> l+1, coarse source on l+1, the one-block tails or coarsest-level
+// relaxations, prolongation l+1 -> l) is one kernel launch covering the blocks of
+// every solve of one model that takes part in it: a block finds its solve by binary search in a
 // prefix table of per-solve block counts and then works exactly as the single-
 // solve kernel does.  One V-cycle of the whole batch is captured once as a CUDA
 // graph and replayed.  Solves that have converged are masked by a device flag
@@ -24,6 +24,7 @@
 #include "mg_internal.h"
 #include "mixed_common.cuh"
 #include "sweep32.cuh"
+#include "tail32.cuh"
 
 namespace mg {
 
@@ -49,6 +50,10 @@ struct BFine {
   float *ub, *tau, *e;
   float* q;            // the finest level's stored neighbour quantity (zeroed with e), or nullptr
 };
+
+// Planes a CTA of the outer residual marches: short, so that a batch of small meshes
+// fills the GPU (two prologue planes each).
+constexpr int kBatchPlanes = 16;
 
 // Level layouts of the batched kernels: the quad kernels take levels whose side
 // is a multiple of 4 (>= 8); others fall back to one cell per thread.
@@ -82,21 +87,22 @@ __global__ void __launch_bounds__(32 * ROWS) kb_smooth(const BDesc* __restrict__
     int seg;
     bool act;
     split_lane(n, n, (long long)b * ROWS + threadIdx.y, threadIdx.x, &r, &seg, &act);
-    if constexpr (K == KFR1 || K == KFR2) {
-      if (d.q) {
-        smooth_split<K, true>(d.lf, n, d.e, d.ub, d.rho, d.S, (int)(r / n), (int)(r % n), seg, act, parity,
-                              threadIdx.x, d.q);
-        return;
-      }
-    }
-    smooth_split<K>(d.lf, n, d.e, d.ub, d.rho, d.S, (int)(r / n), (int)(r % n), seg, act, parity, threadIdx.x);
+    const int i = (int)r / n, j = (int)r - i * n;  // rows: n^2 < 2^31
+    constexpr bool QS = K == KFR1 || K == KFR2;    // these levels store q
+    if (n <= 1024)  // 32-bit cell offsets
+      smooth_split<K, QS, 0, int>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, seg, act, parity, threadIdx.x, d.q);
+    else
+      smooth_split<K, QS>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, seg, act, parity, threadIdx.x, d.q);
     return;
   }
   if (quad_level(n)) {
     const int nbx = ((n >> 2) + 31) / 32;
     const int xb = b % nbx, r = b / nbx, j = r % n, i = (r / n) * ROWS + threadIdx.y;
     if (i >= n) return;  // whole warps
-    smooth_quad<K>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x, parity);
+    if (n <= 1024)
+      smooth_quad<K, false, int>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x, parity);
+    else
+      smooth_quad<K>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x, parity);
     return;
   }
   const long long t = (long long)b * (32 * ROWS) + threadIdx.y * 32 + threadIdx.x;
@@ -117,8 +123,9 @@ static int smooth_blocks(int n, int rows, bool split) {
 
 // Restriction of level l into l+1, d = M(e) - S at 8 children; block (32, 4).
 // Quad levels: ceil(nf/128) x nc x ceil(nc/4) blocks per solve; others: one
-// coarse cell per thread, flat.
-template <int K>
+// coarse cell per thread, flat.  ZR: after pre-smoothing the second colour's defect
+// is zero (restrict_quad, restrict_split_zr).
+template <int K, bool ZR>
 __global__ void __launch_bounds__(128) kb_restrict(const BDesc* __restrict__ D, const int* __restrict__ prefix, int cnt,
                                                    const int* __restrict__ active) {
   const int s = find_slot(prefix, cnt, blockIdx.x);
@@ -130,19 +137,21 @@ __global__ void __launch_bounds__(128) kb_restrict(const BDesc* __restrict__ D, 
     const int nbx = ((nf >> 2) + 31) / 32;
     const int xb = b % nbx, r = b / nbx, J = r % nc, I = (r / nc) * 4 + threadIdx.y;
     if (I >= nc) return;  // whole warps
-    if constexpr (K == KFR1 || K == KFR2) {
-      if (d.split && d.q) {
-        restrict_quad<K, SplitLayout, true>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J,
-                                            xb * 32 + threadIdx.x, threadIdx.x, d.q);
-        return;
+    const int tq = xb * 32 + threadIdx.x, lane = threadIdx.x;
+    constexpr bool QS = K == KFR1 || K == KFR2;  // split levels of these store q
+    if (d.split) {
+      if constexpr (QS && ZR) {
+        if (nf <= 1024) restrict_split_zr<K, int>(d.lf, nf, d.e, d.ub, d.S, d.q, d.ReH, d.eH, d.ubH, d.SH, I, J, tq, lane);
+        else restrict_split_zr<K>(d.lf, nf, d.e, d.ub, d.S, d.q, d.ReH, d.eH, d.ubH, d.SH, I, J, tq, lane);
+      } else {
+        restrict_quad<K, SplitLayout, QS, ZR>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J, tq, lane,
+                                              d.q);
       }
+    } else if (nf <= 1024) {
+      restrict_quad<K, NatLayout32, false, ZR>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J, tq, lane);
+    } else {
+      restrict_quad<K, NatLayout, false, ZR>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J, tq, lane);
     }
-    if (d.split)
-      restrict_quad<K, SplitLayout>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J,
-                                    xb * 32 + threadIdx.x, threadIdx.x);
-    else
-      restrict_quad<K>(d.lf, nf, d.e, d.ub, d.rho, d.S, d.ReH, d.eH, d.ubH, d.SH, I, J, xb * 32 + threadIdx.x,
-                       threadIdx.x);
     return;
   }
   const long long t = (long long)b * 128 + threadIdx.y * 32 + threadIdx.x;
@@ -172,30 +181,45 @@ static int restrict_blocks(int nf) {
   return (int)(((long long)nc * nc * nc + 127) / 128);
 }
 
-// Coarse source on level l (descriptors of level l): S <- M(Re) - S.
+// Coarse source on level l (descriptors of level l): S <- M(Re) - S; block (32, 4).
+// Quad levels: ceil(n/128) x n x n/4 blocks per solve; others: one cell per thread, flat.
 template <int K>
-__global__ void __launch_bounds__(64) kb_fas(const BDesc* __restrict__ D, const int* __restrict__ prefix, int cnt,
-                                             const int* __restrict__ active) {
+__global__ void __launch_bounds__(128) kb_fas(const BDesc* __restrict__ D, const int* __restrict__ prefix, int cnt,
+                                              const int* __restrict__ active) {
   const int s = find_slot(prefix, cnt, blockIdx.x);
   const BDesc& d = D[s];
   if (!active[d.solve]) return;
-  const int n = d.n, nxb = (n + 63) / 64;
+  const int n = d.n;
   const int b = blockIdx.x - prefix[s];
-  const int xb = b % nxb, r = b / nxb, j = r % n, i = r / n;
-  const int k = xb * 64 + threadIdx.x;
-  if (k >= n) return;
-  const size_t t = cidx(n, i, j, k);
+  if (quad_level(n)) {
+    const int nbx = ((n >> 2) + 31) / 32;
+    const int xb = b % nbx, r = b / nbx, j = r % n, i = (r / n) * 4 + threadIdx.y;
+    if (n <= 1024) fas_quad<K, int>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x);
+    else fas_quad<K>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x);
+    return;
+  }
+  const long long t = (long long)b * 128 + threadIdx.y * 32 + threadIdx.x;
+  if (t >= (long long)n * n * n) return;
+  const int k = (int)(t % n), j = (int)((t / n) % n), i = (int)(t / ((long long)n * n));
   d.S[t] = local_M<K>(d.lf, d.ub[t], d.Re[t], d.rho ? d.rho[t] : 1.f, nb_sum_g<K>(d.Re, d.ub, n, i, j, k)) - d.S[t];
+}
+
+static int fas_blocks(int n) {
+  if (quad_level(n)) return (((n >> 2) + 31) / 32) * n * (n / 4);
+  return (int)(((long long)n * n * n + 127) / 128);
 }
 
 // Prolongation-correction of level l from l+1; block (32, 4).  Quad levels:
 // ceil(nf/128) x nf x ceil(nf/4) blocks per solve; others: one fine cell per
 // thread, flat.
-// QK >= 0 (f(R) n = QK): levels with a stored q get it written (prolong_quad),
-// only for the second colour when SO (post-smoothing follows).
-template <bool FR, int QK = -1, bool SO = false>
+// SO (post-smoothing follows): a split finest level has its second colour corrected
+// only (prolong_split2x2_second; CQ's batched levels are not split), for which
+// the blocks are those of the restriction.
+template <int K, bool SO>
 __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, const int* __restrict__ prefix, int cnt,
                                                   const int* __restrict__ active, unsigned long long* guards) {
+  constexpr bool FR = is_fr(K);
+  constexpr int QK = K == KFR1 || K == KFR2 ? K : -1;  // split levels of these store q
   const int s = find_slot(prefix, cnt, blockIdx.x);
   const BDesc& d = D[s];
   if (!active[d.solve]) return;
@@ -203,19 +227,23 @@ __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, c
   const int nf = d.n, nc = nf >> 1;
   const int b = blockIdx.x - prefix[s];
   if (quad_level(nf)) {
-    const int nbx = ((nf >> 2) + 31) / 32;
-    const int xb = b % nbx, r = b / nbx, j = r % nf, i = (r / nf) * 4 + threadIdx.y;
-    if (i >= nf) return;  // whole warps
-    if constexpr (QK >= 0) {
-      if (d.split && d.q) {
-        prolong_quad<FR, SplitLayout, QK, SO>(nc, d.eH, d.ReH, d.ub, d.e, i, j, xb * 32 + threadIdx.x, threadIdx.x,
-                                              guard, d.q);
+    const int nbx = ((nf >> 2) + 31) / 32, xb = b % nbx, r = b / nbx, lane = threadIdx.x, tq = xb * 32 + lane;
+    if constexpr (SO && K != KFR0) {
+      if (d.split) {
+        const int J = r % nc, I = (r / nc) * 4 + threadIdx.y;
+        if (I >= nc) return;  // whole warps
+        if (nf <= 1024)
+          prolong_split2x2_second<QK, false, int>(nc, d.eH, d.ReH, d.ub, d.e, I, J, tq, lane, guard, d.q);
+        else
+          prolong_split2x2_second<QK>(nc, d.eH, d.ReH, d.ub, d.e, I, J, tq, lane, guard, d.q);
         return;
       }
     }
-    if (d.split)
-      prolong_quad<FR, SplitLayout>(nc, d.eH, d.ReH, d.ub, d.e, i, j, xb * 32 + threadIdx.x, threadIdx.x, guard);
-    else prolong_quad<FR>(nc, d.eH, d.ReH, d.ub, d.e, i, j, xb * 32 + threadIdx.x, threadIdx.x, guard);
+    const int j = r % nf, i = (r / nf) * 4 + threadIdx.y;
+    if (i >= nf) return;  // whole warps
+    if (d.split) prolong_quad<FR, SplitLayout, QK>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard, d.q);
+    else if (nf <= 1024) prolong_quad<FR, NatLayout32>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard);
+    else prolong_quad<FR>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard);
     return;
   }
   const long long t = (long long)b * 128 + threadIdx.y * 32 + threadIdx.x;
@@ -240,7 +268,9 @@ __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, c
   d.e[o] = v;
 }
 
-static int prolong_blocks(int nf) {
+// second: the split level's second-colour form.
+static int prolong_blocks(int nf, bool second) {
+  if (second) return restrict_blocks(nf);
   if (quad_level(nf)) return (((nf >> 2) + 31) / 32) * nf * ((nf + 3) / 4);
   return (int)(((long long)nf * nf * nf + 127) / 128);
 }
@@ -264,7 +294,22 @@ __global__ void __launch_bounds__(512) kb_coarse(const BDesc* __restrict__ D, co
     }
 }
 
-// FP64 fine residual of every active solve (tiles of 8 x 32, chunks of 64 planes).
+// The coarsest levels of every solve, one CTA each (tail32.cuh).
+template <int K>
+__global__ void __launch_bounds__(kTailThreads) kb_tail(const TailArgs* __restrict__ args,
+                                                        const int* __restrict__ solve,
+                                                        const int* __restrict__ active) {
+  if (!active[solve[blockIdx.x]]) return;
+  extern __shared__ float tail_sm[];
+  __shared__ TailArgs A;
+  static_assert(sizeof(TailArgs) % 4 == 0, "copied by words");
+  for (int i = threadIdx.x; i < (int)(sizeof(TailArgs) / 4); i += kTailThreads)
+    reinterpret_cast<int*>(&A)[i] = reinterpret_cast<const int*>(args + blockIdx.x)[i];
+  __syncthreads();
+  tail_cycle<K, 2>(A, tail_sm);
+}
+
+// FP64 fine residual of every active solve (tiles of 8 x 32, chunks of kBatchPlanes planes).
 template <int K>
 __global__ void __launch_bounds__(256) kb_outer_residual(const BFine* __restrict__ F, const int* __restrict__ prefix,
                                                          int cnt, const int* __restrict__ active,
@@ -276,11 +321,11 @@ __global__ void __launch_bounds__(256) kb_outer_residual(const BFine* __restrict
   if (active[f.solve]) {
     const int tiles = (f.n / 32) * (f.n / 8);
     if constexpr (K == KCQ) {
-      a = cq_residual_tile<false, 8, 32, false>(f.m, CqSeries{}, 0.0, f.n, 64, f.u, f.src, nullptr, f.ub, f.tau,
+      a = cq_residual_tile<false, 8, 32, false>(f.m, CqSeries{}, 0.0, f.n, kBatchPlanes, f.u, f.src, nullptr, f.ub, f.tau,
                                                 b % tiles, b / tiles);
     } else {
       const FFC c = *f.ffc;
-      a = outer_residual_tile_ff<K, 8, 32, true>(c, f.n, 64, f.u, f.rho, f.ub, f.tau, b % tiles, b / tiles);
+      a = outer_residual_tile_ff<K, 8, 32, true>(c, f.n, kBatchPlanes, f.u, f.rho, f.ub, f.tau, b % tiles, b / tiles);
     }
   }
   if (threadIdx.x == 0) partials[blockIdx.x] = a;
@@ -296,33 +341,61 @@ __global__ void kb_finalize(const BFine* __restrict__ F, const int* __restrict__
   if (threadIdx.x == 0) out[F[s].solve] = a;
 }
 
-// u64 += e and e <- 0 (and the stored q <- 0) for every active solve (fine-cell grid).
+// u64 += e, e <- 0 and the stored q <- 0 for every active solve; a thread takes the
+// cells k = 4w .. 4w + 3 of a row (sides are multiples of 32), which sit at 2w, 2w + 1
+// of the two colours of a split level.
 __global__ void __launch_bounds__(256) kb_apply(const BFine* __restrict__ F, const int* __restrict__ prefix, int cnt,
-                                                const int* __restrict__ active, int clear_only) {
+                                                const int* __restrict__ active) {
   const int s = find_slot(prefix, cnt, blockIdx.x);
   const BFine& f = F[s];
   if (!active[f.solve]) return;
-  const size_t n3 = (size_t)f.n * f.n * f.n;
-  const size_t t = (size_t)(blockIdx.x - prefix[s]) * 256 + threadIdx.x;
-  if (t >= n3) return;
-  // f(R) and symmetron fine levels are split (float-float residual); CQ keeps the natural layout
-  const long long c = f.m.kind == KCQ ? (long long)t
-                                      : split_idx(f.n, (int)(t / ((size_t)f.n * f.n)), (int)((t / f.n) % f.n),
-                                                  (int)(t % f.n));
-  if (!clear_only) f.u[t] += (double)f.e[c];
-  f.e[c] = 0.f;
-  if (f.q) f.q[c] = 0.f;  // Delta w(u, 0)
+  const int n = f.n, w4 = n >> 2, h = n >> 1;
+  const long long t = (long long)(blockIdx.x - prefix[s]) * 256 + threadIdx.x;  // < 2^31: n <= 2048
+  if (t >= (long long)n * n * w4) return;
+  const int row = (int)((unsigned)t / (unsigned)w4), w = (int)t - row * w4;
+  const int i = row / n, j = row - i * n;
+  double* u = f.u + (long long)row * n + 4 * w;
+  float4 e;
+  if (f.m.kind == KCQ) {
+    float4* p = reinterpret_cast<float4*>(f.e + (long long)row * n + 4 * w);
+    e = *p;
+    *p = make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
+    const long long H = (long long)n * n * h, o = (long long)row * h + 2 * w;
+    const long long a = (i + j) & 1 ? H + o : o, b = (i + j) & 1 ? o : H + o;
+    const float2 x = *reinterpret_cast<const float2*>(f.e + a), y = *reinterpret_cast<const float2*>(f.e + b);
+    e = make_float4(x.x, y.x, x.y, y.y);
+    const float2 z = make_float2(0.f, 0.f);
+    *reinterpret_cast<float2*>(f.e + a) = z;
+    *reinterpret_cast<float2*>(f.e + b) = z;
+    if (f.q) {  // Delta w(u, 0)
+      *reinterpret_cast<float2*>(f.q + a) = z;
+      *reinterpret_cast<float2*>(f.q + b) = z;
+    }
+  }
+  if ((uintptr_t)f.u % 16 == 0) {
+    double2* p = reinterpret_cast<double2*>(u);
+    const double2 a = p[0], b = p[1];
+    p[0] = make_double2(a.x + (double)e.x, a.y + (double)e.y);
+    p[1] = make_double2(b.x + (double)e.z, b.y + (double)e.w);
+  } else {
+    u[0] += (double)e.x;
+    u[1] += (double)e.y;
+    u[2] += (double)e.z;
+    u[3] += (double)e.w;
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
 
-struct Phase {            // one batched launch: kind group, descriptor table, block prefix
-  int kind = 0, cnt = 0, blocks = 0;
-  BDesc* d = nullptr;     // device
-  int* prefix = nullptr;  // device, cnt + 1
+struct Phase {                    // one batched launch of one kind
+  int cnt = 0, blocks = 0;
+  size_t d_off = 0, p_off = 0;    // descriptor table and block prefix (cnt + 1) in the batch's tables
 };
+
+constexpr int kBatchKinds = 5;  // model kinds
 
 struct Batch {
   int device = -1;
@@ -347,10 +420,11 @@ struct Batch {
   unsigned long long* h_guards = nullptr;  // pinned host mirror
   int* h_active = nullptr;     // pinned host mirror
   double* h_sums = nullptr;    // pinned host mirror of sums (count) and ssum (count)
-  void* tables = nullptr;      // descriptor tables and prefixes
-  size_t tables_bytes = 0;
+  char* tables = nullptr;      // descriptor tables and prefixes
+  size_t tables_bytes = 0;     // their capacity
   cudaGraphExec_t vexec = nullptr;
-  cudaStream_t cap = nullptr;
+  cudaStream_t cap[kBatchKinds] = {};  // capture streams, one per kind of the batch
+  cudaEvent_t ev[kBatchKinds] = {};
   unsigned long long vsig = 0;
   long long vlaunches = 0;
   int rows = 0;                // autotuned smoother block height (planes per block)
@@ -362,7 +436,10 @@ static std::vector<Batch*> g_batches;
 
 static void free_batch(Batch* b) {
   if (b->vexec) cudaGraphExecDestroy(b->vexec);
-  if (b->cap) cudaStreamDestroy(b->cap);
+  for (int k = 0; k < kBatchKinds; ++k) {
+    if (b->cap[k]) cudaStreamDestroy(b->cap[k]);
+    if (b->ev[k]) cudaEventDestroy(b->ev[k]);
+  }
   if (b->tables) cudaFree(b->tables);
   if (b->base) cudaFree(b->base);
   if (b->h_active) cudaFreeHost(b->h_active);
@@ -419,7 +496,7 @@ static int get_batch(int count, const int* N, const mgglam_params* prm, Batch** 
       o[s].Re[l] = take(c);
       o[s].rho[l] = take(c);
     }
-    total_blocks += (size_t)(N[s] / 32) * (N[s] / 8) * ((N[s] + 63) / 64);
+    total_blocks += (size_t)(N[s] / 32) * (N[s] / 8) * ((N[s] + kBatchPlanes - 1) / kBatchPlanes);
   }
   const size_t o_part = take(std::max<size_t>(total_blocks, kMaxReduceBlocks) * 8);
   const size_t o_sums = take(count * 8), o_ssum = take(count * 8), o_rmean = take(count * 8), o_act = take(count * 4);
@@ -473,46 +550,60 @@ static int get_batch(int count, const int* N, const mgglam_params* prm, Batch** 
     default: { constexpr int KK = KCQ; CALL; } break;                   \
   }
 
-struct Plan {
-  // per level l: phases for kinds present; smooth/restrict/prolong over solves with
-  // last level > l; fas over level l+1 of the same solves; coarse for last level == l
-  struct LevelPhases {
-    std::vector<Phase> smooth, restrict_, fas, prolong, coarse;
+// The launches of one kind's solves: per level l the phases of the solves that go
+// below l (smoothing, restriction, prolongation, and the source on l + 1, which a
+// tail forms itself), the solves whose V-cycle ends on l with a coarsest
+// relaxation, and those whose rest runs as a tail.
+struct KindPlan {
+  int kind = 0;
+  struct L {
+    Phase smooth, restrict_, fas, prolong, coarse;
   };
-  std::vector<LevelPhases> lv;
-  std::vector<Phase> outer;  // fine levels, per kind (tiled residual)
-  std::vector<Phase> apply;  // fine levels, per kind (256 cells per block)
-  std::vector<BFine*> fine_desc;
-  std::vector<int*> fine_prefix;
+  std::vector<L> lv;
+  int tails = 0;
+  size_t tail_off = 0, tail_solve_off = 0, tail_smem = 0;
+  Phase outer, apply;
+  size_t fine_off = 0;
 };
 
-// Build all descriptor tables in one device allocation.
+struct Plan {
+  std::vector<KindPlan> kinds;
+};
+
+// First level of solve s's one-block tail (tail32.cuh), or -1.
+static int batch_tail(const Batch::S& v) {
+  int n[kMaxLevels];
+  for (int l = 0; l < v.nlev; ++l) n[l] = v.N >> l;
+  for (int l = 1; l < v.nlev; ++l)
+    if (tail_fits(n, v.nlev, l)) return l;
+  return -1;
+}
+
+// Build all descriptor tables and bring them to the device (one copy, into memory
+// the batch keeps).
 static int build_plan(Batch* B, const std::vector<ModelDev>& models, const std::vector<std::vector<LevelF>>& lfs,
                       const std::vector<const float*>& rho_in, double* const* field, const mgglam_params* prm,
-                      bool need_rho_any, int rows, Plan* P, cudaStream_t st) {
-  (void)need_rho_any;
-  (void)prm;
+                      int rows, Plan* P, cudaStream_t st) {
   const int count = B->count;
-  int Lmax = 0;
-  for (auto& v : B->sv) Lmax = std::max(Lmax, v.nlev);
-  // host staging buffer of descriptors + prefixes
   std::vector<char> host;
-  struct Pending { Phase* ph; size_t d_off, p_off; };
-  std::vector<Pending> pend;
-  auto align = [&](size_t x) { return (x + 255) & ~(size_t)255; };
-  auto add_phase = [&](Phase& ph, const std::vector<BDesc>& ds, const std::vector<int>& blocks) {
-    ph.cnt = (int)ds.size();
-    size_t d_off = align(host.size());
-    host.resize(d_off + ds.size() * sizeof(BDesc));
-    memcpy(host.data() + d_off, ds.data(), ds.size() * sizeof(BDesc));
-    size_t p_off = align(host.size());
-    host.resize(p_off + (ds.size() + 1) * sizeof(int));
-    int* pf = (int*)(host.data() + p_off);
-    int acc = 0;
-    for (size_t i = 0; i < ds.size(); ++i) { pf[i] = acc; acc += blocks[i]; }
-    pf[ds.size()] = acc;
-    ph.blocks = acc;
-    pend.push_back({&ph, d_off, p_off});
+  auto put = [&](const void* data, size_t bytes) {
+    const size_t off = (host.size() + 255) & ~(size_t)255;
+    host.resize(off + bytes);
+    memcpy(host.data() + off, data, bytes);
+    return off;
+  };
+  auto phase = [&](size_t d_off, const std::vector<int>& blocks) {
+    Phase ph;
+    ph.cnt = (int)blocks.size();
+    ph.d_off = d_off;
+    std::vector<int> pf(blocks.size() + 1);
+    for (size_t i = 0; i < blocks.size(); ++i) pf[i + 1] = pf[i] + blocks[i];
+    ph.blocks = pf.back();
+    ph.p_off = put(pf.data(), pf.size() * sizeof(int));
+    return ph;
+  };
+  auto rho_needed = [&](int s) {
+    return models[s].kind == KSYM || (models[s].kind == KCQ && models[s].keep_exp);
   };
   auto desc = [&](int s, int l) {
     const Batch::S& v = B->sv[s];
@@ -526,8 +617,7 @@ static int build_plan(Batch* B, const std::vector<ModelDev>& models, const std::
     d.e = v.e[l];
     d.ub = v.ub[l];
     d.S = v.S32[l];
-    const bool rho_needed = models[s].kind == KSYM || (models[s].kind == KCQ && models[s].keep_exp);
-    d.rho = rho_needed ? v.rho32[l] : nullptr;
+    d.rho = rho_needed(s) ? v.rho32[l] : nullptr;
     d.Re = v.Re[l];
     if (l + 1 < v.nlev) {
       d.eH = v.e[l + 1];
@@ -537,89 +627,82 @@ static int build_plan(Batch* B, const std::vector<ModelDev>& models, const std::
     }
     return d;
   };
-  P->lv.assign(Lmax, {});
   std::vector<int> kinds;
   for (auto& m : models)
     if (std::find(kinds.begin(), kinds.end(), m.kind) == kinds.end()) kinds.push_back(m.kind);
-  for (int l = 0; l < Lmax; ++l) {
-    for (int kind : kinds) {
-      std::vector<BDesc> sm, fa, co;
-      std::vector<int> bsm, bre, bfa, bpr, bco;
-      for (int s = 0; s < count; ++s) {
-        if (models[s].kind != kind) continue;
-        const int last = B->sv[s].nlev - 1;
-        const int n = B->sv[s].N >> l;
-        if (l < last) {
-          sm.push_back(desc(s, l));
-          bsm.push_back(smooth_blocks(n, rows, l == 0 && models[s].kind != KCQ));
-          bre.push_back(restrict_blocks(n));
-          bpr.push_back(prolong_blocks(n));
-          fa.push_back(desc(s, l + 1));
-          bfa.push_back(((n / 2 + 63) / 64) * (n / 2) * (n / 2));
-        } else if (l == last) {
-          co.push_back(desc(s, l));
-          bco.push_back(1);
-        }
-      }
-      if (!sm.empty()) {
-        Phase a, b, c, d;
-        a.kind = b.kind = c.kind = d.kind = kind;
-        P->lv[l].smooth.push_back(a);
-        P->lv[l].restrict_.push_back(b);
-        P->lv[l].fas.push_back(c);
-        P->lv[l].prolong.push_back(d);
-      }
-      if (!co.empty()) {
-        Phase e;
-        e.kind = kind;
-        P->lv[l].coarse.push_back(e);
-      }
-    }
-  }
-  // second pass now that the vectors no longer move: fill tables
-  for (int l = 0; l < Lmax; ++l) {
-    int is = 0, ic = 0;
-    for (int kind : kinds) {
-      std::vector<BDesc> sm, fa, co;
-      std::vector<int> bsm, bre, bfa, bpr, bco;
-      for (int s = 0; s < count; ++s) {
-        if (models[s].kind != kind) continue;
-        const int last = B->sv[s].nlev - 1;
-        const int n = B->sv[s].N >> l;
-        if (l < last) {
-          sm.push_back(desc(s, l));
-          bsm.push_back(smooth_blocks(n, rows, l == 0 && models[s].kind != KCQ));
-          bre.push_back(restrict_blocks(n));
-          bpr.push_back(prolong_blocks(n));
-          fa.push_back(desc(s, l + 1));
-          bfa.push_back(((n / 2 + 63) / 64) * (n / 2) * (n / 2));
-        } else if (l == last) {
-          co.push_back(desc(s, l));
-          bco.push_back(1);
-        }
-      }
-      if (!sm.empty()) {
-        add_phase(P->lv[l].smooth[is], sm, bsm);
-        add_phase(P->lv[l].restrict_[is], sm, bre);
-        add_phase(P->lv[l].fas[is], fa, bfa);
-        add_phase(P->lv[l].prolong[is], sm, bpr);
-        ++is;
-      }
-      if (!co.empty()) add_phase(P->lv[l].coarse[ic++], co, bco);
-    }
-  }
-  // fine-level tables for the FP64 kernels (outer residual tiles; apply in 256-cell blocks)
-  std::vector<std::vector<BFine>> fk(kinds.size());
-  P->outer.assign(kinds.size(), {});
-  P->apply.assign(kinds.size(), {});
-  std::vector<size_t> fine_off(kinds.size()), fpo(kinds.size()), fpa(kinds.size());
+  P->kinds.assign(kinds.size(), {});
   for (size_t g = 0; g < kinds.size(); ++g) {
-    std::vector<int> bo, ba;
+    KindPlan& G = P->kinds[g];
+    G.kind = kinds[g];
+    std::vector<int> own, tail(count), last(count);
+    int Lmax = 0;
     for (int s = 0; s < count; ++s) {
-      if (models[s].kind != kinds[g]) continue;
+      if (models[s].kind != G.kind) continue;
+      own.push_back(s);
+      tail[s] = batch_tail(B->sv[s]);
+      last[s] = tail[s] > 0 ? tail[s] : B->sv[s].nlev - 1;  // the level whose V-cycle is one launch
+      Lmax = std::max(Lmax, last[s] + 1);
+    }
+    G.lv.assign(Lmax, {});
+    for (int l = 0; l < Lmax; ++l) {
+      std::vector<BDesc> go, src, end;
+      std::vector<int> bsm, bre, bfa, bpr;
+      for (int s : own) {
+        const int n = B->sv[s].N >> l;
+        const bool split = l == 0 && G.kind != KCQ;
+        if (l < last[s]) {
+          go.push_back(desc(s, l));
+          bsm.push_back(smooth_blocks(n, rows, split));
+          bre.push_back(restrict_blocks(n));
+          bpr.push_back(prolong_blocks(n, split && G.kind != KFR0 && prm[0].nu2 >= 1));
+          if (l + 1 != tail[s]) {
+            src.push_back(desc(s, l + 1));
+            bfa.push_back(fas_blocks(n / 2));
+          }
+        } else if (l == last[s] && tail[s] < 0) {
+          end.push_back(desc(s, l));
+        }
+      }
+      KindPlan::L& L = G.lv[l];
+      if (!go.empty()) {
+        const size_t d = put(go.data(), go.size() * sizeof(BDesc));
+        L.smooth = phase(d, bsm);
+        L.restrict_ = phase(d, bre);
+        L.prolong = phase(d, bpr);
+      }
+      if (!src.empty()) L.fas = phase(put(src.data(), src.size() * sizeof(BDesc)), bfa);
+      if (!end.empty()) L.coarse = phase(put(end.data(), end.size() * sizeof(BDesc)), std::vector<int>(end.size(), 1));
+    }
+    std::vector<TailArgs> ta;
+    std::vector<int> ts;
+    std::vector<BFine> fine;
+    std::vector<int> bo, ba;
+    for (int s : own) {
+      const Batch::S& v = B->sv[s];
+      if (tail[s] > 0) {
+        TailArgs A;
+        memset(&A, 0, sizeof(A));
+        const int t = tail[s];
+        A.T = v.nlev - t;
+        for (int m = 0; m < A.T; ++m) {
+          A.n[m] = v.N >> (t + m);
+          A.lf[m] = lfs[s][t + m];
+          A.rho[m] = rho_needed(s) ? v.rho32[t + m] : nullptr;
+          A.zr[m] = G.kind != KCQ || cq_linear(lfs[s][t + m]);
+        }
+        A.e = v.e[t];
+        A.ub = v.ub[t];
+        A.S = v.S32[t];
+        A.nu1 = prm[0].nu1;
+        A.nu2 = prm[0].nu2;
+        A.coarse_sweeps = prm[0].coarse_sweeps;
+        A.guard = B->guards + s;
+        G.tail_smem = std::max(G.tail_smem, tail_layout(A));
+        ta.push_back(A);
+        ts.push_back(s);
+      }
       BFine f;
       memset(&f, 0, sizeof(f));
-      const Batch::S& v = B->sv[s];
       f.n = v.N;
       f.solve = s;
       f.m = models[s];
@@ -630,102 +713,110 @@ static int build_plan(Batch* B, const std::vector<ModelDev>& models, const std::
       f.ub = v.ub[0];
       f.tau = v.S32[0];
       f.e = v.e[0];
-      f.q = (models[s].kind == KFR1 || models[s].kind == KFR2) ? v.q0 : nullptr;
-      fk[g].push_back(f);
-      bo.push_back((v.N / 32) * (v.N / 8) * ((v.N + 63) / 64));
-      ba.push_back((int)(((size_t)v.N * v.N * v.N + 255) / 256));
+      f.q = (G.kind == KFR1 || G.kind == KFR2) ? v.q0 : nullptr;
+      fine.push_back(f);
+      bo.push_back((v.N / 32) * (v.N / 8) * ((v.N + kBatchPlanes - 1) / kBatchPlanes));
+      ba.push_back((int)(((size_t)v.N * v.N * (v.N / 4) + 255) / 256));
     }
-    P->outer[g].kind = P->apply[g].kind = kinds[g];
-    // stage BFine tables with the same layout helper (reinterpret as bytes)
-    size_t d_off = align(host.size());
-    host.resize(d_off + fk[g].size() * sizeof(BFine));
-    memcpy(host.data() + d_off, fk[g].data(), fk[g].size() * sizeof(BFine));
-    fine_off[g] = d_off;
-    auto put_prefix = [&](const std::vector<int>& bl, Phase& ph) {
-      size_t p_off = align(host.size());
-      host.resize(p_off + (bl.size() + 1) * sizeof(int));
-      int* pf = (int*)(host.data() + p_off);
-      int acc = 0;
-      for (size_t i = 0; i < bl.size(); ++i) { pf[i] = acc; acc += bl[i]; }
-      pf[bl.size()] = acc;
-      ph.blocks = acc;
-      ph.cnt = (int)bl.size();
-      return p_off;
-    };
-    fpo[g] = put_prefix(bo, P->outer[g]);
-    fpa[g] = put_prefix(ba, P->apply[g]);
+    G.tails = (int)ta.size();
+    if (G.tails) {
+      G.tail_off = put(ta.data(), ta.size() * sizeof(TailArgs));
+      G.tail_solve_off = put(ts.data(), ts.size() * sizeof(int));
+    }
+    G.fine_off = put(fine.data(), fine.size() * sizeof(BFine));
+    G.outer = phase(G.fine_off, bo);
+    G.apply = phase(G.fine_off, ba);
   }
-  // upload
-  if (B->tables) cudaFree(B->tables);
-  B->tables = nullptr;
-  if (cudaMalloc(&B->tables, host.size() + 256) != cudaSuccess) {
-    cudaGetLastError();
-    return MGGLAM_ERR_OOM;
+  if (B->tables_bytes < host.size()) {
+    if (B->tables) cudaFree(B->tables);
+    B->tables = nullptr;
+    B->tables_bytes = 0;
+    const size_t cap = host.size() + host.size() / 2;  // other models of the same meshes fit too
+    if (cudaMalloc((void**)&B->tables, cap) != cudaSuccess) {
+      cudaGetLastError();
+      return MGGLAM_ERR_OOM;
+    }
+    B->tables_bytes = cap;
   }
-  B->tables_bytes = host.size();
   MG_CUDA_TRY(cudaMemcpyAsync(B->tables, host.data(), host.size(), cudaMemcpyHostToDevice, st));
   MG_CUDA_TRY(cudaStreamSynchronize(st));
-  char* tb = (char*)B->tables;
-  for (auto& pd : pend) {
-    pd.ph->d = (BDesc*)(tb + pd.d_off);
-    pd.ph->prefix = (int*)(tb + pd.p_off);
-  }
-  P->fine_desc.resize(kinds.size());
-  P->fine_prefix.resize(kinds.size());
-  for (size_t g = 0; g < kinds.size(); ++g) {
-    P->fine_desc[g] = (BFine*)(tb + fine_off[g]);
-    P->outer[g].prefix = (int*)(tb + fpo[g]);
-    P->apply[g].prefix = (int*)(tb + fpa[g]);
-  }
   return MGGLAM_OK;
 }
 
-static void launch_smooth_phase(const Phase& ph, int rows, const int* active, int parity, cudaStream_t st) {
+static const BDesc* descs(const Batch* B, const Phase& ph) { return (const BDesc*)(B->tables + ph.d_off); }
+static const int* prefix_of(const Batch* B, const Phase& ph) { return (const int*)(B->tables + ph.p_off); }
+
+static void launch_smooth_phase(const Batch* B, int kind, const Phase& ph, int rows, int parity, cudaStream_t st) {
   if (ph.blocks == 0) return;
+  const BDesc* d = descs(B, ph);
+  const int* pf = prefix_of(B, ph);
   switch (rows) {
-    case 2: MG_BDISPATCH(ph.kind, (kb_smooth<KK, 2><<<ph.blocks, dim3(32, 2), 0, st>>>(ph.d, ph.prefix, ph.cnt, active, parity))); break;
-    case 8: MG_BDISPATCH(ph.kind, (kb_smooth<KK, 8><<<ph.blocks, dim3(32, 8), 0, st>>>(ph.d, ph.prefix, ph.cnt, active, parity))); break;
-    default: MG_BDISPATCH(ph.kind, (kb_smooth<KK, 4><<<ph.blocks, dim3(32, 4), 0, st>>>(ph.d, ph.prefix, ph.cnt, active, parity))); break;
+    case 2: MG_BDISPATCH(kind, (kb_smooth<KK, 2><<<ph.blocks, dim3(32, 2), 0, st>>>(d, pf, ph.cnt, B->active, parity))); break;
+    case 8: MG_BDISPATCH(kind, (kb_smooth<KK, 8><<<ph.blocks, dim3(32, 8), 0, st>>>(d, pf, ph.cnt, B->active, parity))); break;
+    default: MG_BDISPATCH(kind, (kb_smooth<KK, 4><<<ph.blocks, dim3(32, 4), 0, st>>>(d, pf, ph.cnt, B->active, parity))); break;
   }
   note_launch(1);
 }
 
-// One V-cycle of every active solve.
-static void batch_vcycle(const Plan& P, const int* active, unsigned long long* guards, const mgglam_params& prm,
-                         int rows, cudaStream_t st) {
-  const int Lmax = (int)P.lv.size();
+template <int K>
+static void launch_batch_restrict(const Batch* B, const Phase& p, bool relaxed, cudaStream_t st) {
+  // CQ's one Newton step leaves a defect in general
+  if (K != KCQ && relaxed)
+    kb_restrict<K, K != KCQ><<<p.blocks, dim3(32, 4), 0, st>>>(descs(B, p), prefix_of(B, p), p.cnt, B->active);
+  else
+    kb_restrict<K, false><<<p.blocks, dim3(32, 4), 0, st>>>(descs(B, p), prefix_of(B, p), p.cnt, B->active);
+}
+
+template <int K>
+static void launch_batch_tail(const Batch* B, const KindPlan& G, cudaStream_t st) {
+  kb_tail<K><<<G.tails, kTailThreads, G.tail_smem, st>>>((const TailArgs*)(B->tables + G.tail_off),
+                                                         (const int*)(B->tables + G.tail_solve_off), B->active);
+}
+
+template <int K>
+static int allow_batch_tail() {
+  MG_CUDA_TRY(cudaFuncSetAttribute(kb_tail<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
+  return MGGLAM_OK;
+}
+
+// One V-cycle of every active solve of one kind.
+static void batch_vcycle(const Batch* B, const KindPlan& G, const mgglam_params& prm, cudaStream_t st) {
+  const int Lmax = (int)G.lv.size();
+  const dim3 b4(32, 4);
   for (int l = 0; l < Lmax; ++l) {
-    const auto& L = P.lv[l];
-    for (size_t g = 0; g < L.smooth.size(); ++g) {
-      for (int s = 0; s < prm.nu1; ++s)
-        for (int par = 0; par < 2; ++par) launch_smooth_phase(L.smooth[g], rows, active, par, st);
-      const Phase& r = L.restrict_[g];
-      MG_BDISPATCH(r.kind, (kb_restrict<KK><<<r.blocks, dim3(32, 4), 0, st>>>(r.d, r.prefix, r.cnt, active)));
-      const Phase& f = L.fas[g];
-      MG_BDISPATCH(f.kind, (kb_fas<KK><<<f.blocks, 64, 0, st>>>(f.d, f.prefix, f.cnt, active)));
-      note_launch(2);
+    const KindPlan::L& L = G.lv[l];
+    for (int s = 0; s < 2 * prm.nu1; ++s) launch_smooth_phase(B, G.kind, L.smooth, B->rows, s & 1, st);
+    if (L.restrict_.blocks) {
+      MG_BDISPATCH(G.kind, (launch_batch_restrict<KK>(B, L.restrict_, prm.nu1 > 0, st)));
+      note_launch(1);
     }
-    for (const Phase& c : L.coarse) {
-      MG_BDISPATCH(c.kind, (kb_coarse<KK><<<c.cnt, 512, 0, st>>>(c.d, active, prm.coarse_sweeps)));
+    const Phase& f = L.fas;
+    if (f.blocks) {
+      MG_BDISPATCH(G.kind, (kb_fas<KK><<<f.blocks, b4, 0, st>>>(descs(B, f), prefix_of(B, f), f.cnt, B->active)));
+      note_launch(1);
+    }
+    if (L.coarse.cnt) {
+      MG_BDISPATCH(G.kind, (kb_coarse<KK><<<L.coarse.cnt, 512, 0, st>>>(descs(B, L.coarse), B->active, prm.coarse_sweeps)));
       note_launch(1);
     }
   }
-  for (int l = Lmax - 2; l >= 0; --l) {
-    const auto& L = P.lv[l];
-    for (size_t g = 0; g < L.prolong.size(); ++g) {
-      const Phase& p = L.prolong[g];
-      const bool so = prm.nu2 >= 1;  // the same for every solve of the batch
-      const dim3 b4(32, 4);
-      if (p.kind == KFR1 && so) kb_prolong<true, KFR1, true><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      else if (p.kind == KFR1) kb_prolong<true, KFR1><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      else if (p.kind == KFR2 && so) kb_prolong<true, KFR2, true><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      else if (p.kind == KFR2) kb_prolong<true, KFR2><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      else if (is_fr(p.kind)) kb_prolong<true><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      else kb_prolong<false><<<p.blocks, b4, 0, st>>>(p.d, p.prefix, p.cnt, active, guards);
-      note_launch(1);
-      for (int s = 0; s < prm.nu2; ++s)
-        for (int par = 0; par < 2; ++par) launch_smooth_phase(L.smooth[g], rows, active, par, st);
+  if (G.tails) {
+    MG_BDISPATCH(G.kind, (launch_batch_tail<KK>(B, G, st)));
+    note_launch(1);
+  }
+  for (int l = Lmax - 1; l >= 0; --l) {
+    const KindPlan::L& L = G.lv[l];
+    const Phase& p = L.prolong;
+    if (!p.blocks) continue;
+    if (prm.nu2 >= 1) {
+      MG_BDISPATCH(G.kind, (kb_prolong<KK, true><<<p.blocks, b4, 0, st>>>(descs(B, p), prefix_of(B, p), p.cnt, B->active,
+                                                                          B->guards)));
+    } else {
+      MG_BDISPATCH(G.kind, (kb_prolong<KK, false><<<p.blocks, b4, 0, st>>>(descs(B, p), prefix_of(B, p), p.cnt, B->active,
+                                                                           B->guards)));
     }
+    note_launch(1);
+    for (int s = 0; s < 2 * prm.nu2; ++s) launch_smooth_phase(B, G.kind, L.smooth, B->rows, s & 1, st);
   }
 }
 
@@ -754,9 +845,15 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
       k_ff_consts<<<1, 32, 0, st>>>(models[s], n3, B->rmean + s, B->ffc + s);
     }
     const bool split = models[s].kind != KCQ;
-    if (split) k_density_norm32_split<<<stream_grid(n3), kThreads, 0, st>>>(rho[s], v.N, B->rmean + s, v.rho32[0]);
-    else k_density_norm32<<<stream_grid(n3), kThreads, 0, st>>>(rho[s], n3, B->rmean + s, v.rho32[0]);
-    for (int l = 1; l < v.nlev; ++l) {
+    // the density pyramid, where the operator takes it
+    const bool rho_needed = models[s].kind == KSYM || (models[s].kind == KCQ && models[s].keep_exp);
+    if (!rho_needed) {
+    } else if (split) {
+      k_density_norm32_split<<<stream_grid(n3), kThreads, 0, st>>>(rho[s], v.N, B->rmean + s, v.rho32[0]);
+    } else {
+      k_density_norm32<<<stream_grid(n3), kThreads, 0, st>>>(rho[s], n3, B->rmean + s, v.rho32[0]);
+    }
+    for (int l = 1; l < v.nlev && rho_needed; ++l) {
       const int nc = v.N >> l;
       if (l == 1 && split)
         k_restrict32_from_split<<<dim3((nc + 63) / 64, nc, nc), 64, 0, st>>>(v.N, v.rho32[0], v.rho32[1]);
@@ -769,23 +866,21 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
     k_finalize_sum32<<<1, 1024, 0, st>>>(B->partials, stream_grid(n3), B->ssum + s);
     MG_CUDA_TRY(cudaMemsetAsync(v.e[0], 0, (size_t)n3 * 4, st));
     MG_CUDA_TRY(cudaMemsetAsync(v.q0, 0, (size_t)n3 * 4, st));  // Delta w(u, 0) = 0
-    note_launch(5 + v.nlev);
+    note_launch(4 + (rho_needed ? v.nlev : 0));
   }
   Plan P;
-  if ((rc = build_plan(B, models, lfs, std::vector<const float*>(rho, rho + count), field, prm, false,
-                       B->rows ? B->rows : 4, &P, st)))
-    return rc;
-  const int ng = (int)P.outer.size();
+  const std::vector<const float*> rho_in(rho, rho + count);
+  if ((rc = build_plan(B, models, lfs, rho_in, field, prm, B->rows ? B->rows : 4, &P, st))) return rc;
+  auto fine_of = [&](const KindPlan& G) { return (const BFine*)(B->tables + G.fine_off); };
   auto outer_residual = [&]() -> int {
-    for (int g = 0; g < ng; ++g) {
-      const Phase& o = P.outer[g];
-      // partial slots: each group's blocks start after the previous groups'
-      int base = 0;
-      for (int h = 0; h < g; ++h) base += P.outer[h].blocks;
-      MG_BDISPATCH(o.kind, (kb_outer_residual<KK><<<o.blocks, 256, 0, st>>>(P.fine_desc[g], o.prefix, o.cnt,
+    int base = 0;  // partial slots: each kind's blocks after the previous ones'
+    for (const KindPlan& G : P.kinds) {
+      const Phase& o = G.outer;
+      MG_BDISPATCH(G.kind, (kb_outer_residual<KK><<<o.blocks, 256, 0, st>>>(fine_of(G), prefix_of(B, o), o.cnt,
                                                                              B->active, B->partials + base)));
-      kb_finalize<<<o.cnt, 256, 0, st>>>(P.fine_desc[g], o.prefix, o.cnt, B->partials + base, B->sums);
+      kb_finalize<<<o.cnt, 256, 0, st>>>(fine_of(G), prefix_of(B, o), o.cnt, B->partials + base, B->sums);
       note_launch(2);
+      base += o.blocks;
     }
     MG_CUDA_TRY(cudaMemcpyAsync(B->h_sums, B->sums, count * 8, cudaMemcpyDeviceToHost, st));
     MG_CUDA_TRY(cudaMemcpyAsync(B->h_sums + count, B->ssum, count * 8, cudaMemcpyDeviceToHost, st));
@@ -804,17 +899,18 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
     float best_ms = 1e30f;
     for (int cand : {2, 4, 8}) {
       Plan Pt;
-      if ((rc = build_plan(B, models, lfs, std::vector<const float*>(rho, rho + count), field, prm, false, cand, &Pt, st)))
-        return rc;
+      if ((rc = build_plan(B, models, lfs, rho_in, field, prm, cand, &Pt, st))) return rc;
       for (int s = 0; s < count; ++s) B->h_active[s] = 1;
       MG_CUDA_TRY(cudaMemcpyAsync(B->active, B->h_active, count * 4, cudaMemcpyHostToDevice, st));
       cudaEvent_t e0, e1;
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
-      for (const Phase& ph : Pt.lv[0].smooth) launch_smooth_phase(ph, cand, B->active, 0, st);  // warm
+      auto pass = [&](int parity) {
+        for (const KindPlan& G : Pt.kinds) launch_smooth_phase(B, G.kind, G.lv[0].smooth, cand, parity, st);
+      };
+      pass(0);  // warm
       cudaEventRecord(e0, st);
-      for (int rep = 0; rep < 3; ++rep)
-        for (const Phase& ph : Pt.lv[0].smooth) launch_smooth_phase(ph, cand, B->active, rep & 1, st);
+      for (int rep = 0; rep < 3; ++rep) pass(rep & 1);
       cudaEventRecord(e1, st);
       cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -830,9 +926,7 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
       MG_CUDA_TRY(cudaMemsetAsync(B->sv[s].e[0], 0, bytes, st));
       MG_CUDA_TRY(cudaMemsetAsync(B->sv[s].q0, 0, bytes, st));
     }
-    if ((rc = build_plan(B, models, lfs, std::vector<const float*>(rho, rho + count), field, prm, false, B->rows, &P,
-                         st)))
-      return rc;
+    if ((rc = build_plan(B, models, lfs, rho_in, field, prm, B->rows, &P, st))) return rc;
   }
   std::vector<double> snorm(count), eps(count);
   std::vector<mgglam_stats> lst(count);
@@ -845,29 +939,52 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
     lst[s].resid0 = eps[s];
     lst[s].resid_hist[0] = eps[s];
   }
-  // graph of one batched V-cycle (captured per plan signature)
-  if (!B->cap && cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking) != cudaSuccess) return MGGLAM_ERR_CUDA;
-  unsigned long long sig = 1469598103934665603ull;
-  auto mix = [&](const void* p, size_t n) {
-    const unsigned char* bb = (const unsigned char*)p;
-    for (size_t i = 0; i < n; ++i) sig = (sig ^ bb[i]) * 1099511628211ull;
-  };
-  for (int s = 0; s < count; ++s) {
-    mix(lfs[s].data(), lfs[s].size() * sizeof(LevelF));
-    mix(&models[s].kind, sizeof(int));
-    mix(&field[s], sizeof(double*));
+  // Graph of one batched V-cycle: the kinds' chains of launches are branches of it,
+  // so that one kind's small levels, bound by latency, run beside another's.  All a
+  // launch bakes in is its table's place and block count; the constants and buffers
+  // are in the tables, so other parameters or fields of the same meshes replay the
+  // same graph.
+  for (size_t k = 0; k < P.kinds.size(); ++k) {
+    if (!B->cap[k] && cudaStreamCreateWithFlags(&B->cap[k], cudaStreamNonBlocking) != cudaSuccess) return MGGLAM_ERR_CUDA;
+    if (!B->ev[k] && cudaEventCreateWithFlags(&B->ev[k], cudaEventDisableTiming) != cudaSuccess) return MGGLAM_ERR_CUDA;
+    if (P.kinds[k].tails) {
+      MG_BDISPATCH(P.kinds[k].kind, rc = allow_batch_tail<KK>());
+      if (rc) return rc;
+    }
   }
-  const int shape[4] = {prm[0].nu1, prm[0].nu2, prm[0].coarse_sweeps, B->rows};
-  mix(shape, sizeof(shape));
-  mix(&B->tables, sizeof(void*));
+  unsigned long long sig = 1469598103934665603ull;
+  auto mix = [&](unsigned long long v) { sig = (sig ^ v) * 1099511628211ull; };
+  auto mix_phase = [&](const Phase& p) {
+    mix(p.cnt);
+    mix(p.blocks);
+    mix(p.d_off);
+    mix(p.p_off);
+  };
+  for (const KindPlan& G : P.kinds) {
+    mix(G.kind);
+    mix(G.tails);
+    mix(G.tail_off);
+    mix(G.tail_solve_off);
+    mix(G.tail_smem);
+    mix(G.lv.size());
+    for (const KindPlan::L& L : G.lv)
+      for (const Phase* p : {&L.smooth, &L.restrict_, &L.fas, &L.prolong, &L.coarse}) mix_phase(*p);
+  }
+  for (int v : {prm[0].nu1, prm[0].nu2, prm[0].coarse_sweeps, B->rows}) mix((unsigned long long)v);
+  mix((unsigned long long)(uintptr_t)B->tables);
   if (!(B->vexec && B->vsig == sig)) {
     if (B->vexec) { cudaGraphExecDestroy(B->vexec); B->vexec = nullptr; }
     const long long n0 = launch_count();
     cudaGraph_t g = nullptr;
-    bool ok = cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    bool ok = cudaStreamBeginCapture(B->cap[0], cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-      batch_vcycle(P, B->active, B->guards, prm[0], B->rows, B->cap);
-      ok = cudaStreamEndCapture(B->cap, &g) == cudaSuccess && g;
+      ok = cudaEventRecord(B->ev[0], B->cap[0]) == cudaSuccess;
+      for (size_t k = 1; k < P.kinds.size() && ok; ++k) ok = cudaStreamWaitEvent(B->cap[k], B->ev[0], 0) == cudaSuccess;
+      for (size_t k = 0; k < P.kinds.size() && ok; ++k) batch_vcycle(B, P.kinds[k], prm[0], B->cap[k]);
+      for (size_t k = 1; k < P.kinds.size() && ok; ++k)
+        ok = cudaEventRecord(B->ev[k], B->cap[k]) == cudaSuccess &&
+             cudaStreamWaitEvent(B->cap[0], B->ev[k], 0) == cudaSuccess;
+      ok = cudaStreamEndCapture(B->cap[0], &g) == cudaSuccess && g && ok;
     }
     B->vlaunches = launch_count() - n0;
     note_launch((int)-B->vlaunches);
@@ -894,11 +1011,6 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
     }
     if (!any) break;
     MG_CUDA_TRY(cudaMemcpyAsync(B->active, B->h_active, count * 4, cudaMemcpyHostToDevice, st));
-    // e <- 0 on the fine levels of the active solves
-    for (int g = 0; g < ng; ++g) {
-      kb_apply<<<P.apply[g].blocks, 256, 0, st>>>(P.fine_desc[g], P.apply[g].prefix, P.apply[g].cnt, B->active, 1);
-      note_launch(1);
-    }
     int inner = prm[0].inner_cycles;
     if (inner <= 0) {
       const double lr = log(rho_est);
@@ -914,8 +1026,8 @@ int solve_batch(int count, const mgglam_params* prm, const double* a, const floa
       for (int s = 0; s < count; ++s)
         if (B->h_active[s]) ++lst[s].cycles;
     }
-    for (int g = 0; g < ng; ++g) {
-      kb_apply<<<P.apply[g].blocks, 256, 0, st>>>(P.fine_desc[g], P.apply[g].prefix, P.apply[g].cnt, B->active, 0);
+    for (const KindPlan& G : P.kinds) {  // which leaves e at zero for the next step
+      kb_apply<<<G.apply.blocks, 256, 0, st>>>(fine_of(G), prefix_of(B, G.apply), G.apply.cnt, B->active);
       note_launch(1);
     }
     ++outer;

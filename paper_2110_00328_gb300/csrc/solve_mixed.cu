@@ -616,7 +616,7 @@ static int fas_source(const MixedCtx& C, int l, cudaStream_t st) {
 // Coarse-grid correction seen from the finest level: the FAS source on level 1
 // and the cycle(s) on levels >= 1 (V: one; W: two W; F: F then V), enqueued directly.
 static int coarse_part_direct(const MixedCtx& C, cudaStream_t st) {
-  int rc = fas_source(C, 1, st);
+  int rc = C.tail_level == 1 ? MGGLAM_OK : fas_source(C, 1, st);  // the tail forms its own
   if (rc) return rc;
   const int mode = C.prm->cycle;
   rc = vcycle32(C, 1, st, mode);
@@ -649,6 +649,7 @@ static unsigned long long coarse_signature(const MixedCtx& C) {
 // ping-pong buffers as it found them, the kernels are enqueued directly.
 static int coarse_part(const MixedCtx& C, cudaStream_t st) {
   Workspace* ws = C.ws;
+  if (C.tail_level == 1) return coarse_part_direct(C, st);  // one kernel: a graph would only add its own launch
   const unsigned long long sig = coarse_signature(C);
   if (!(ws->coarse_exec && ws->coarse_sig == sig)) {
     if (ws->coarse_exec) {
@@ -693,8 +694,8 @@ static int coarse_part(const MixedCtx& C, cudaStream_t st) {
 
 // Levels tail_level .. coarsest in one CTA (tail32.cuh).
 template <int K>
-static void launch_tail_t(const TailArgs& A, cudaStream_t st) {
-  k_tail32<K><<<1, kTailThreads, tail_smem_bytes(A), st>>>(A);
+static void launch_tail_t(const TailArgs& A, size_t smem, cudaStream_t st) {
+  (tail_cpt(A.n[0]) == 2 ? k_tail32<K, 2> : k_tail32<K, 1>)<<<1, kTailThreads, smem, st>>>(A);
 }
 
 static int launch_tail(const MixedCtx& C, int l, cudaStream_t st) {
@@ -706,6 +707,7 @@ static int launch_tail(const MixedCtx& C, int l, cudaStream_t st) {
     A.n[m] = ws->lev[l + m].n;
     A.lf[m] = C.lf[l + m];
     A.rho[m] = C.need_rho ? ws->lev[l + m].rho32 : nullptr;
+    A.zr[m] = C.m.kind != KCQ || cq_linear(C.lf[l + m]);
   }
   A.e = ws->lev[l].e;
   A.ub = ws->lev[l].ub;
@@ -714,18 +716,21 @@ static int launch_tail(const MixedCtx& C, int l, cudaStream_t st) {
   A.nu2 = C.prm->nu2;
   A.coarse_sweeps = C.prm->coarse_sweeps;
   A.guard = C.guard;
-  MG_DISPATCH32(C.m.kind, (launch_tail_t<KK>(A, st)));
+  const size_t smem = tail_layout(A);
+  MG_DISPATCH32(C.m.kind, (launch_tail_t<KK>(A, smem, st)));
   return MGGLAM_OK;
 }
 
-// The tail's shared memory can exceed the 48 KB default (at most ~94 KB).
-static void tail_allow_smem() {
-  const int bytes = 96 * 1024;
-  cudaFuncSetAttribute(k_tail32<KFR0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(k_tail32<KFR1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(k_tail32<KFR2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(k_tail32<KSYM>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(k_tail32<KCQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+// The tail's shared memory exceeds the 48 KB default (at most 120 KB).
+template <int K>
+static void tail_allow_smem_t() {
+  cudaFuncSetAttribute(k_tail32<K, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+  cudaFuncSetAttribute(k_tail32<K, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+}
+
+static int tail_allow_smem(int kind) {
+  MG_DISPATCH32(kind, (tail_allow_smem_t<KK>(), note_launch(-1)));
+  return MGGLAM_OK;
 }
 
 // The restriction after pre-smoothing (ZR) of a level in layout FL, per model kind.
@@ -887,7 +892,7 @@ static int vcycle32(const MixedCtx& C, int l, cudaStream_t st, int mode) {
     prof_begin(PC_COARSE_LEVELS, st, 0.0);
     if ((rc = coarse_part(C, st))) return rc;
   } else {
-    if ((rc = fas_source(C, l + 1, st))) return rc;
+    if (l + 1 != C.tail_level && (rc = fas_source(C, l + 1, st))) return rc;  // the tail forms its own
     if ((rc = vcycle32(C, l + 1, st, mode))) return rc;
     if (mode != 0 && (rc = vcycle32(C, l + 1, st, mode == 2 ? 2 : 0))) return rc;
   }
@@ -1094,13 +1099,12 @@ int solve_mixed(const mgglam_params* prm, double a, const float* rho, int N, dou
   const L2Scope l2s(q_window_begin(C));
   C.l2 = &l2s.w;
   C.tail_level = -1;  // the one-block tail runs V-cycles only
-  const long long tail_cells = prm->tail_cells == 0 ? 512 : (prm->tail_cells > kTailMaxCells ? kTailMaxCells : prm->tail_cells);
-  for (int l = 1; l < C.ws->nlev && tail_cells > 0 && prm->cycle == 0; ++l)
-    if ((long long)C.ws->lev[l].n3 <= tail_cells && C.ws->nlev - l <= kTailMaxLevels) {
-      C.tail_level = l;
-      break;
-    }
-  if (C.tail_level > 0) tail_allow_smem();
+  const long long tail_cells = prm->tail_cells == 0 ? kTailMaxCells : prm->tail_cells;
+  int sides[kMaxLevels];
+  for (int l = 0; l < C.ws->nlev; ++l) sides[l] = C.ws->lev[l].n;
+  for (int l = 1; l < C.ws->nlev && prm->cycle == 0 && C.tail_level < 0; ++l)
+    if ((long long)C.ws->lev[l].n3 <= tail_cells && tail_fits(sides, C.ws->nlev, l)) C.tail_level = l;
+  if (C.tail_level > 0) tail_allow_smem(C.m.kind);
   Workspace* ws = C.ws;
   for (int l = 0; l < ws->nlev; ++l) C.lf[l] = make_levelf(C.m, ws->lev[l].h);
   Level& F = ws->lev[0];
