@@ -90,10 +90,12 @@ typedef struct {
                          one pass per colour (measured faster at 256^3: the kernel is bound
                          by instruction issue, and the extra launches cost more than the
                          DRAM traffic they save) */
-  int tail_cells;     /* MIXED: the coarsest levels, from the first level (below the finest)
-                         with at most this many cells, run as one thread block with the
-                         levels in shared memory (same arithmetic, fewer launches).
-                         0 (default) = 4096, the most; < 0 = off */
+  int tail_cells;     /* MIXED: the coarsest levels, from the first level with at most this
+                         many cells, run as one kernel with the levels in shared memory
+                         (same arithmetic, fewer launches): a cluster of thread blocks from
+                         a level of side 20 .. 32 (the finest: 8 .. 32), else one block from
+                         the first level below the finest with at most 4096 cells.
+                         0 (default) = 32768, the most; < 0 = off */
   int cycle;          /* multigrid cycle: 0 (default) V, 1 F, 2 W (Sec. 3.2.1; each level
                          recurses once (V), twice (W), or F then V (F)) */
   int fmg;            /* 1: full-multigrid start (f(R), symmetron): the first cycle solves

@@ -74,6 +74,7 @@ struct Workspace {
   cudaGraphExec_t coarse_exec = nullptr;
   unsigned long long coarse_sig = 0;
   long long coarse_launches = 0;
+  unsigned cluster_asked = 0, cluster_ok = 0;  // per model kind: whether the clustered tail can run
 };
 
 // Slots of Workspace::scalars.

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float
 
 // The deposit of np particles on acc: of an M x M x ... array (M^2 a divisor of np) of
 // at least two bricks an SM and half a particle a cell -- below that the window's
-// zeroing and flush, eight cells a particle, cost more than the atomics they save --
+// zeroing and flush, four cells a particle, cost more than the atomics they save --
 // in a mesh of at least the window's longest side brick by brick, else in the order
 // of the array.  lattice: M, or 0.
 static int launch_deposit(const float* pos, long long np, long long lattice, int N, unsigned long long* acc,

@@ -325,7 +325,7 @@ struct MixedCtx {
   bool split;         // the finest level in the red-black split layout
   bool ff_resid;      // fine residual in float-float (f(R), symmetron) rather than FP64 (CQ)
   CqSeries cq;        // CQ: the potential's series
-  int tail_level;     // first level (>= 1) run by the one-block tail kernel, or -1
+  int tail_level;     // first level run by the tail kernel (0: of a cluster tail only), or -1
   float* qs;          // split f(R) n = 1, 2: the finest level's stored neighbour quantity, else nullptr
   unsigned long long* guard;  // positivity-guard replacements of this solve (workspace scalar)
   const struct L2Window* l2 = nullptr;  // persisting L2 window over qs for the colour passes, or nullptr
@@ -698,39 +698,129 @@ static void launch_tail_t(const TailArgs& A, size_t smem, cudaStream_t st) {
   (tail_cpt(A.n[0]) == 2 ? k_tail32<K, 2> : k_tail32<K, 1>)<<<1, kTailThreads, smem, st>>>(A);
 }
 
-static int launch_tail(const MixedCtx& C, int l, cudaStream_t st) {
+static TailArgs tail_args(const MixedCtx& C, int l) {
   Workspace* ws = C.ws;
   TailArgs A;
   memset(&A, 0, sizeof(A));
-  A.T = ws->nlev - l;
+  A.T = ws->nlev - l;  // 0: none (the last two levels are a cluster's own)
   for (int m = 0; m < A.T; ++m) {
     A.n[m] = ws->lev[l + m].n;
     A.lf[m] = C.lf[l + m];
     A.rho[m] = C.need_rho ? ws->lev[l + m].rho32 : nullptr;
     A.zr[m] = C.m.kind != KCQ || cq_linear(C.lf[l + m]);
   }
-  A.e = ws->lev[l].e;
-  A.ub = ws->lev[l].ub;
-  A.S = ws->lev[l].S32;
+  if (A.T) {
+    A.e = ws->lev[l].e;
+    A.ub = ws->lev[l].ub;
+    A.S = ws->lev[l].S32;
+  }
   A.nu1 = C.prm->nu1;
   A.nu2 = C.prm->nu2;
   A.coarse_sweeps = C.prm->coarse_sweeps;
   A.guard = C.guard;
+  return A;
+}
+
+// One cluster for the levels from l on (k_tail32_cluster): V-cycles one after the other.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  ClusterLaunch(size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClusterCtas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+};
+
+template <int K>
+static cudaError_t launch_cluster_t(const ClusterArgs& A, size_t smem, cudaStream_t st) {
+  ClusterLaunch c(smem, st);
+  return cudaLaunchKernelEx(&c.cfg, k_tail32_cluster<K>, A);
+}
+
+static int launch_cluster(const MixedCtx& C, int l, int cycles, cudaStream_t st) {
+  Level& L = C.ws->lev[l];
+  ClusterArgs A;
+  memset(&A, 0, sizeof(A));
+  A.in = tail_args(C, l + 2);
+  A.n = L.n;
+  for (int m = 0; m < 2; ++m) {
+    A.lf[m] = C.lf[l + m];
+    A.rho[m] = C.need_rho ? C.ws->lev[l + m].rho32 : nullptr;
+    A.zr[m] = C.m.kind != KCQ || cq_linear(C.lf[l + m]);
+  }
+  A.finest = l == 0;
+  A.split = A.finest && C.split;
+  A.second = A.finest && C.prm->nu2 >= 1 && second_colour_only(C);
+  A.cycles = cycles;
+  A.e = L.e;
+  A.ub = L.ub;
+  A.S = L.S32;
+  if (A.finest && C.fresh) {
+    A.fresh = *C.fresh;
+    *C.fresh = false;
+  }
+  const size_t smem = cluster_layout(A);
+  MG_DISPATCH32(C.m.kind, MG_CUDA_TRY(launch_cluster_t<KK>(A, smem, st)));
+  return MGGLAM_OK;
+}
+
+static int launch_tail(const MixedCtx& C, int l, cudaStream_t st) {
+  if (l == 0 || C.ws->lev[l].n > kTailMaxSide) return launch_cluster(C, l, 1, st);
+  TailArgs A = tail_args(C, l);
   const size_t smem = tail_layout(A);
   MG_DISPATCH32(C.m.kind, (launch_tail_t<KK>(A, smem, st)));
   return MGGLAM_OK;
 }
 
-// The tail's shared memory exceeds the 48 KB default (at most 120 KB).
+// The tails' shared memory exceeds the 48 KB default (at most 120 KB), a cluster of 16 CTAs is beyond the
+// portable size of 8.
 template <int K>
 static void tail_allow_smem_t() {
   cudaFuncSetAttribute(k_tail32<K, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
   cudaFuncSetAttribute(k_tail32<K, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+  cudaFuncSetAttribute(k_tail32_cluster<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+  cudaFuncSetAttribute(k_tail32_cluster<K>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
 static int tail_allow_smem(int kind) {
   MG_DISPATCH32(kind, (tail_allow_smem_t<KK>(), note_launch(-1)));
   return MGGLAM_OK;
+}
+
+// Whether a cluster finds 16 SMs it can run on together (a partition of the GPU may not
+// have them); asked once a workspace and kind.
+template <int K>
+static bool cluster_runs_t() {
+  ClusterLaunch c(128 * 1024, nullptr);
+  int clusters = 0;
+  const bool ok = cudaOccupancyMaxActiveClusters(&clusters, k_tail32_cluster<K>, &c.cfg) == cudaSuccess && clusters > 0;
+  cudaGetLastError();
+  return ok;
+}
+
+static bool cluster_runs(Workspace* ws, int kind) {
+  const unsigned bit = 1u << kind;
+  if (!(ws->cluster_asked & bit)) {
+    tail_allow_smem(kind);
+    bool ok = false;
+    switch (kind) {
+      case KFR0: ok = cluster_runs_t<KFR0>(); break;
+      case KFR1: ok = cluster_runs_t<KFR1>(); break;
+      case KFR2: ok = cluster_runs_t<KFR2>(); break;
+      case KSYM: ok = cluster_runs_t<KSYM>(); break;
+      default: ok = cluster_runs_t<KCQ>(); break;
+    }
+    ws->cluster_asked |= bit;
+    if (ok) ws->cluster_ok |= bit;
+  }
+  return ws->cluster_ok & bit;
 }
 
 // The restriction after pre-smoothing (ZR) of a level in layout FL, per model kind.
@@ -1098,13 +1188,22 @@ int solve_mixed(const mgglam_params* prm, double a, const float* rho, int N, dou
   C.guard = guard_of(C.ws);
   const L2Scope l2s(q_window_begin(C));
   C.l2 = &l2s.w;
-  C.tail_level = -1;  // the one-block tail runs V-cycles only
-  const long long tail_cells = prm->tail_cells == 0 ? kTailMaxCells : prm->tail_cells;
+  // The tail runs V-cycles only: from a level of side 20 .. 32 (the finest 8 .. 32) as a
+  // cluster, else from the first coarse level of at most 16^3 cells as one block.
+  // (A thread holds one pair of the cluster's level, which ends at 32^3; a 16^3 tail is
+  // 18 us as one block, whose way down to it the cluster would not shorten.)  A forced
+  // fused sweep keeps the levels it fits.
+  C.tail_level = -1;
+  const long long tail_cells =
+      prm->tail_cells != 0 ? prm->tail_cells : prm->sweep_chunk > 0 ? kTailMaxCells : kClusterCells;
   int sides[kMaxLevels];
   for (int l = 0; l < C.ws->nlev; ++l) sides[l] = C.ws->lev[l].n;
-  for (int l = 1; l < C.ws->nlev && prm->cycle == 0 && C.tail_level < 0; ++l)
-    if ((long long)C.ws->lev[l].n3 <= tail_cells && tail_fits(sides, C.ws->nlev, l)) C.tail_level = l;
-  if (C.tail_level > 0) tail_allow_smem(C.m.kind);
+  for (int l = 0; l < C.ws->nlev && prm->cycle == 0 && C.tail_level < 0; ++l)
+    if ((long long)C.ws->lev[l].n3 <= tail_cells &&
+        ((l > 0 && tail_fits(sides, C.ws->nlev, l)) ||
+         (cluster_fits(sides, C.ws->nlev, l) && cluster_runs(C.ws, C.m.kind))))
+      C.tail_level = l;
+  if (C.tail_level >= 0) tail_allow_smem(C.m.kind);
   Workspace* ws = C.ws;
   for (int l = 0; l < ws->nlev; ++l) C.lf[l] = make_levelf(C.m, ws->lev[l].h);
   Level& F = ws->lev[0];
@@ -1185,8 +1284,13 @@ int solve_mixed(const mgglam_params* prm, double a, const float* rho, int N, dou
       if (C.qs) MG_CUDA_TRY(cudaMemsetAsync(C.qs, 0, F.n3 * sizeof(float), st));  // Delta w(u, 0) = 0
     }
     fresh = fresh_ok && !fmg;
-    for (int c = 0; c < inner && cyc < prm->max_cycles; ++c, ++cyc, ++done)
-      if ((rc = (fmg && c == 0) ? fmg_start32(C, st) : vcycle32(C, 0, st, C.prm->cycle))) return rc;
+    for (int c = 0; c < inner && cyc < prm->max_cycles; ++c, ++cyc, ++done) {
+      if (C.tail_level == 0 && !(fmg && c == 0)) {  // the outer step's remaining cycles in one launch
+        const int k = inner - c < prm->max_cycles - cyc ? inner - c : prm->max_cycles - cyc;
+        if ((rc = launch_cluster(C, 0, k, st))) return rc;
+        c += k - 1, cyc += k - 1, done += k - 1;
+      } else if ((rc = (fmg && c == 0) ? fmg_start32(C, st) : vcycle32(C, 0, st, C.prm->cycle))) return rc;
+    }
     prof_begin(PC_APPLY_CORR, st, 20.0 * n3);
     const bool vec = C.split && (uintptr_t)field % 16 == 0;  // the split layout has n % 32 == 0
     if (vec && bg_pending)
