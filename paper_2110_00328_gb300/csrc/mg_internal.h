@@ -159,11 +159,12 @@ void release_batches();
 // ---- particles (particles.cu) ----
 int deposit_cic(const float* pos, long long np, int N, float* rho, cudaStream_t st);
 void forget_static_deposit_address();
+// lattice: the side M of the M x M x ... array the particles are in the order of, 0: none, -1: np = M^3 decides.
 int gather_force(const ModelDev& m, int kind, int n_fr, const mgglam_params* prm,
                  const double* field, int N, const float* pos, long long np, float* force,
-                 double prefactor, cudaStream_t st);
+                 double prefactor, cudaStream_t st, long long lattice = -1);
 int gather_chunk(const ModelDev& m, int kind, const mgglam_params* prm, int N, const float* pos, long long np,
-                 float* force, double prefactor, cudaStream_t st);
+                 float* force, double prefactor, cudaStream_t st, long long lattice);
 int deposit_cic_host(const float* pos_host, float* pos_dev, long long np, int N, float* rho, int chunks,
                      cudaStream_t st);
 int gather_force_host(const ModelDev& m, int kind, const mgglam_params* prm, const double* field, int N,
