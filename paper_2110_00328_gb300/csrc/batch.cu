@@ -97,12 +97,13 @@ __global__ void __launch_bounds__(32 * ROWS) kb_smooth(const BDesc* __restrict__
   }
   if (quad_level(n)) {
     const int nbx = ((n >> 2) + 31) / 32;
-    const int xb = b % nbx, r = b / nbx, j = r % n, i = (r / n) * ROWS + threadIdx.y;
+    const int xb = b % nbx, r = b / nbx, nr = n / quad_rows(n), i = (r / nr) * ROWS + threadIdx.y;
     if (i >= n) return;  // whole warps
+    const QuadLane<true> ql(n, r % nr, xb, threadIdx.x);
     if (n <= 1024)
-      smooth_quad<K, false, int>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x, parity);
+      smooth_quad<K, false, int>(d.lf, n, d.e, d.ub, d.rho, d.S, i, ql.j, ql.tq, threadIdx.x, parity);
     else
-      smooth_quad<K>(d.lf, n, d.e, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x, parity);
+      smooth_quad<K>(d.lf, n, d.e, d.ub, d.rho, d.S, i, ql.j, ql.tq, threadIdx.x, parity);
     return;
   }
   const long long t = (long long)b * (32 * ROWS) + threadIdx.y * 32 + threadIdx.x;
@@ -117,7 +118,7 @@ __global__ void __launch_bounds__(32 * ROWS) kb_smooth(const BDesc* __restrict__
 
 static int smooth_blocks(int n, int rows, bool split) {
   if (split) return (int)((split_warps(n, n) + rows - 1) / rows);
-  if (quad_level(n)) return (((n >> 2) + 31) / 32) * n * ((n + rows - 1) / rows);
+  if (quad_level(n)) return (((n >> 2) + 31) / 32) * (n / quad_rows(n)) * ((n + rows - 1) / rows);
   return (int)(((long long)(n >> 1) * n * n + 32 * rows - 1) / (32 * rows));
 }
 
@@ -135,9 +136,10 @@ __global__ void __launch_bounds__(128) kb_restrict(const BDesc* __restrict__ D, 
   const int b = blockIdx.x - prefix[s];
   if (quad_level(nf)) {
     const int nbx = ((nf >> 2) + 31) / 32;
-    const int xb = b % nbx, r = b / nbx, J = r % nc, I = (r / nc) * 4 + threadIdx.y;
+    const int xb = b % nbx, r = b / nbx, nr = nc / quad_rows(nf), I = (r / nr) * 4 + threadIdx.y;
     if (I >= nc) return;  // whole warps
-    const int tq = xb * 32 + threadIdx.x, lane = threadIdx.x;
+    const QuadLane<> ql(nf, r % nr, xb, threadIdx.x);
+    const int J = ql.j, tq = ql.tq, lane = threadIdx.x;
     constexpr bool QS = K == KFR1 || K == KFR2;  // split levels of these store q
     if (d.split) {
       if constexpr (QS && ZR) {
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(128) kb_restrict(const BDesc* __restrict__ D, 
 
 static int restrict_blocks(int nf) {
   const int nc = nf >> 1;
-  if (quad_level(nf)) return (((nf >> 2) + 31) / 32) * nc * ((nc + 3) / 4);
+  if (quad_level(nf)) return (((nf >> 2) + 31) / 32) * (nc / quad_rows(nf)) * ((nc + 3) / 4);
   return (int)(((long long)nc * nc * nc + 127) / 128);
 }
 
@@ -193,9 +195,10 @@ __global__ void __launch_bounds__(128) kb_fas(const BDesc* __restrict__ D, const
   const int b = blockIdx.x - prefix[s];
   if (quad_level(n)) {
     const int nbx = ((n >> 2) + 31) / 32;
-    const int xb = b % nbx, r = b / nbx, j = r % n, i = (r / n) * 4 + threadIdx.y;
-    if (n <= 1024) fas_quad<K, int>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x);
-    else fas_quad<K>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, j, xb * 32 + threadIdx.x, threadIdx.x);
+    const int xb = b % nbx, r = b / nbx, nr = n / quad_rows(n), i = (r / nr) * 4 + threadIdx.y;
+    const QuadLane<> ql(n, r % nr, xb, threadIdx.x);
+    if (n <= 1024) fas_quad<K, int>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, ql.j, ql.tq, threadIdx.x);
+    else fas_quad<K>(d.lf, n, d.Re, d.ub, d.rho, d.S, i, ql.j, ql.tq, threadIdx.x);
     return;
   }
   const long long t = (long long)b * 128 + threadIdx.y * 32 + threadIdx.x;
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(128) kb_fas(const BDesc* __restrict__ D, const
 }
 
 static int fas_blocks(int n) {
-  if (quad_level(n)) return (((n >> 2) + 31) / 32) * n * (n / 4);
+  if (quad_level(n)) return (((n >> 2) + 31) / 32) * (n / quad_rows(n)) * (n / 4);
   return (int)(((long long)n * n * n + 127) / 128);
 }
 
@@ -227,11 +230,13 @@ __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, c
   const int nf = d.n, nc = nf >> 1;
   const int b = blockIdx.x - prefix[s];
   if (quad_level(nf)) {
-    const int nbx = ((nf >> 2) + 31) / 32, xb = b % nbx, r = b / nbx, lane = threadIdx.x, tq = xb * 32 + lane;
+    const int nbx = ((nf >> 2) + 31) / 32, xb = b % nbx, r = b / nbx, lane = threadIdx.x, per = quad_rows(nf);
     if constexpr (SO && K != KFR0) {
       if (d.split) {
-        const int J = r % nc, I = (r / nc) * 4 + threadIdx.y;
+        const int nr = nc / per, I = (r / nr) * 4 + threadIdx.y;
         if (I >= nc) return;  // whole warps
+        const QuadLane<> ql(nf, r % nr, xb, lane);
+        const int J = ql.j, tq = ql.tq;
         if (nf <= 1024)
           prolong_split2x2_second<QK, false, int>(nc, d.eH, d.ReH, d.ub, d.e, I, J, tq, lane, guard, d.q);
         else
@@ -239,8 +244,10 @@ __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, c
         return;
       }
     }
-    const int j = r % nf, i = (r / nf) * 4 + threadIdx.y;
+    const int nr = nf / per, i = (r / nr) * 4 + threadIdx.y;
     if (i >= nf) return;  // whole warps
+    const QuadLane<> ql(nf, r % nr, xb, lane);
+    const int j = ql.j, tq = ql.tq;
     if (d.split) prolong_quad<FR, SplitLayout, QK>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard, d.q);
     else if (nf <= 1024) prolong_quad<FR, NatLayout32>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard);
     else prolong_quad<FR>(nc, d.eH, d.ReH, d.ub, d.e, i, j, tq, lane, guard);
@@ -271,7 +278,7 @@ __global__ void __launch_bounds__(128) kb_prolong(const BDesc* __restrict__ D, c
 // second: the split level's second-colour form.
 static int prolong_blocks(int nf, bool second) {
   if (second) return restrict_blocks(nf);
-  if (quad_level(nf)) return (((nf >> 2) + 31) / 32) * nf * ((nf + 3) / 4);
+  if (quad_level(nf)) return (((nf >> 2) + 31) / 32) * (nf / quad_rows(nf)) * ((nf + 3) / 4);
   return (int)(((long long)nf * nf * nf + 127) / 128);
 }
 

@@ -171,7 +171,7 @@ __device__ __forceinline__ void restrict_quad(const LevelF& f, int nf, const flo
       const float4 q = Q[a][b];
       float qm = __shfl_up_sync(0xffffffffu, q.w, 1);
       float qp = __shfl_down_sync(0xffffffffu, q.x, 1);
-      if (lane == 0) qm = q1(i0 + a, j0 + b, k0 == 0 ? nf - 1 : k0 - 1);
+      if (lane == 0 || tq == 0) qm = q1(i0 + a, j0 + b, k0 == 0 ? nf - 1 : k0 - 1);
       if (lane == 31 || tq + 1 >= nq) qp = q1(i0 + a, j0 + b, k0 + 4 == nf ? 0 : k0 + 4);
       const float4 ni = a == 0 ? qi[0][b] : Q[0][b];   // i - 1
       const float4 pi = a == 0 ? Q[1][b] : qi[1][b];   // i + 1
@@ -255,7 +255,7 @@ __device__ __forceinline__ void fas_quad(const LevelF& f, int n, const float* __
   }
   float qm = __shfl_up_sync(0xffffffffu, q.w, 1);
   float qp = __shfl_down_sync(0xffffffffu, q.x, 1);
-  if (lane == 0) {
+  if (lane == 0 || tq == 0) {
     const IT c = c0 + (k0 == 0 ? n - 1 : -1);
     qm = nbq<K>(FR ? ub[c] : 0.f, Re[c]);
   }
@@ -336,7 +336,7 @@ __device__ __forceinline__ void restrict_split_zr(const LevelF& f, int nf, const
       const float2 q = Q[a][b];
       float qm = __shfl_up_sync(0xffffffffu, q.y, 1);
       float qp = __shfl_down_sync(0xffffffffu, q.x, 1);
-      if (p == 0 && lane == 0) qm = q1[row(i0 + a, j0 + b) + (m0 == 0 ? h - 1 : -1)];
+      if (p == 0 && (lane == 0 || tq == 0)) qm = q1[row(i0 + a, j0 + b) + (m0 == 0 ? h - 1 : -1)];
       if (p == 1 && (lane == 31 || tq + 1 >= nq)) qp = q1[row(i0 + a, j0 + b) + (m0 + 2 == h ? 2 - h : 2)];
       const float k0s = p ? q.x + q.y : qm + q.x;
       const float k1s = p ? q.y + qp : q.x + q.y;
@@ -404,7 +404,7 @@ __device__ __forceinline__ void prolong_quad(int nc, const float* __restrict__ e
   const float Ry = 9.f * A.y + 3.f * (B.y + C.y) + D.y;
   float Rm = __shfl_up_sync(0xffffffffu, Ry, 1);    // coarse k = K0 - 1
   float Rp = __shfl_down_sync(0xffffffffu, Rx, 1);  // coarse k = K0 + 2
-  if (lane == 0) {
+  if (lane == 0 || tq == 0) {
     const int Km = K0 == 0 ? nc - 1 : K0 - 1;
     Rm = 9.f * d1(rA, Km) + 3.f * (d1(rB, Km) + d1(rC, Km)) + d1(rD, Km);
   }
@@ -485,7 +485,7 @@ __device__ __forceinline__ void prolong_split2x2_second(int nc, const float* __r
   const int Km = K0 == 0 ? nc - 1 : K0 - 1, Kp = K0 + 2 == nc ? 0 : K0 + 2;
   const int Iv[3] = {I == 0 ? nc - 1 : I - 1, I, I + 1 == nc ? 0 : I + 1};
   const int Jv[3] = {J == 0 ? nc - 1 : J - 1, J, J + 1 == nc ? 0 : J + 1};
-  const bool edge_m = lane == 0, edge_p = lane == 31 || tq + 1 >= nq;
+  const bool edge_m = lane == 0 || tq == 0, edge_p = lane == 31 || tq + 1 >= nq;
   // coarse differences eH - Re of the nine rows at K0, K0+1 (and K0-1, K0+2 at the row ends)
   float2 d[3][3];
   float dm[3][3], dp[3][3];

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(64) k_smooth32(LevelF f, int n, float* __restr
 }
 
 // Quad version (levels with n % 4 == 0) on the planes i0 .. i0+np-1 (mod n):
-// block (32, 4) = four rows (i, j), grid (ceil(n/128), n, ceil(np/4)).
+// block (32, 4) = four planes i, grid (ceil(n/128), n / quad_rows, ceil(np/4)).
 template <int K, bool WD = false, typename IT = long long>
 __global__ void __launch_bounds__(128) k_smooth32q(LevelF f, int n, float* __restrict__ e,
                                                    const float* __restrict__ ub, const float* __restrict__ rho,
@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(128) k_smooth32q(LevelF f, int n, float* __res
   if (z >= np) return;  // whole warps: z is uniform in a warp
   int i = i0 + z;
   if (i >= n) i -= n;
-  smooth_quad<K, WD, IT>(f, n, e, ub, rho, S, i, blockIdx.y, blockIdx.x * 32 + threadIdx.x, threadIdx.x, parity,
-                         Re, D);
+  const QuadLane<true> ql(n, blockIdx.y, blockIdx.x, threadIdx.x);
+  smooth_quad<K, WD, IT>(f, n, e, ub, rho, S, i, ql.j, ql.tq, threadIdx.x, parity, Re, D);
 }
 
 template <int K>
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(128) k_residual_restrict32(LevelF f, int nf, c
 }
 
 // Quad versions (fine side % 4 == 0): block (32, 4), lanes along k; FL is the
-// fine level's layout.  Restriction: grid (ceil(nf/128), nc [J], ceil(nc/4) [I]).
+// fine level's layout.  Restriction: grid (ceil(nf/128), nc / quad_rows(nf) [J], ceil(nc/4) [I]).
 template <int K, class FL = NatLayout, bool QH = false, bool ZR = false>
 __global__ void __launch_bounds__(128) k_residual_restrict32q(LevelF f, int nf, const float* __restrict__ e,
                                                               const float* __restrict__ ub,
@@ -142,19 +142,20 @@ __global__ void __launch_bounds__(128) k_residual_restrict32q(LevelF f, int nf, 
                                                               const float* __restrict__ qf) {
   const int I = blockIdx.z * 4 + threadIdx.y;
   if (I >= (nf >> 1)) return;  // whole warps
-  restrict_quad<K, FL, QH, ZR>(f, nf, e, ub, rho, S, Re, eH, ubH, SH, I, blockIdx.y, blockIdx.x * 32 + threadIdx.x,
-                               threadIdx.x, qf);
+  const QuadLane<> ql(nf, blockIdx.y, blockIdx.x, threadIdx.x);
+  restrict_quad<K, FL, QH, ZR>(f, nf, e, ub, rho, S, Re, eH, ubH, SH, I, ql.j, ql.tq, threadIdx.x, qf);
 }
 
-// Prolongation: grid (ceil(nf/128), nf [j], nf/4 [i]).
+// Prolongation: grid (ceil(nf/128), nf / quad_rows(nf) [j], nf/4 [i]).
 template <bool FR, class FL = NatLayout, int QK = -1, bool SECOND_ONLY = false>
 __global__ void __launch_bounds__(128) k_prolong_correct32q(int nc, const float* __restrict__ eH,
                                                             const float* __restrict__ Re,
                                                             const float* __restrict__ ub, float* __restrict__ ef,
                                                             unsigned long long* guard,
                                                             float* __restrict__ qf = nullptr) {
-  prolong_quad<FR, FL, QK, SECOND_ONLY>(nc, eH, Re, ub, ef, blockIdx.z * 4 + threadIdx.y, blockIdx.y,
-                                        blockIdx.x * 32 + threadIdx.x, threadIdx.x, guard, qf);
+  const QuadLane<> ql(2 * nc, blockIdx.y, blockIdx.x, threadIdx.x);
+  prolong_quad<FR, FL, QK, SECOND_ONLY>(nc, eH, Re, ub, ef, blockIdx.z * 4 + threadIdx.y, ql.j, ql.tq, threadIdx.x,
+                                        guard, qf);
 }
 
 // Second-colour prolongation on a split finest level with stored q, four fine
@@ -166,8 +167,8 @@ __global__ void __launch_bounds__(128) k_prolong32_split2x2(int nc, const float*
                                                             float* __restrict__ qf) {
   const int I = blockIdx.z * 4 + threadIdx.y;
   if (I >= nc) return;  // whole warps
-  prolong_split2x2_second<QK, DD, IT>(nc, eH, Re, ub, ef, I, blockIdx.y, blockIdx.x * 32 + threadIdx.x,
-                                      threadIdx.x, guard, qf);
+  const QuadLane<> ql(2 * nc, blockIdx.y, blockIdx.x, threadIdx.x);
+  prolong_split2x2_second<QK, DD, IT>(nc, eH, Re, ub, ef, I, ql.j, ql.tq, threadIdx.x, guard, qf);
 }
 
 // Restriction after pre-smoothing on a split finest level with stored q, the
@@ -180,17 +181,17 @@ __global__ void __launch_bounds__(128) k_restrict32_split_zr(LevelF f, int nf, c
                                                              float* __restrict__ ubH, float* __restrict__ SH) {
   const int I = blockIdx.z * 4 + threadIdx.y;
   if (I >= (nf >> 1)) return;  // whole warps
-  restrict_split_zr<K, IT>(f, nf, e, ub, S, qf, Re, eH, ubH, SH, I, blockIdx.y, blockIdx.x * 32 + threadIdx.x,
-                           threadIdx.x);
+  const QuadLane<> ql(nf, blockIdx.y, blockIdx.x, threadIdx.x);
+  restrict_split_zr<K, IT>(f, nf, e, ub, S, qf, Re, eH, ubH, SH, I, ql.j, ql.tq, threadIdx.x);
 }
 
-// FAS source, four cells per lane (n % 4 == 0, n >= 8): grid (ceil(n/128), n, n/4).
+// FAS source, four cells per lane (n % 4 == 0, n >= 8): grid (ceil(n/128), n / quad_rows, n/4).
 template <int K, typename IT = long long>
 __global__ void __launch_bounds__(128) k_fas_source32q(LevelF f, int n, const float* __restrict__ Re,
                                                        const float* __restrict__ ub, const float* __restrict__ rho,
                                                        float* __restrict__ S) {
-  fas_quad<K, IT>(f, n, Re, ub, rho, S, blockIdx.z * 4 + threadIdx.y, blockIdx.y, blockIdx.x * 32 + threadIdx.x,
-              threadIdx.x);
+  const QuadLane<> ql(n, blockIdx.y, blockIdx.x, threadIdx.x);
+  fas_quad<K, IT>(f, n, Re, ub, rho, S, blockIdx.z * 4 + threadIdx.y, ql.j, ql.tq, threadIdx.x);
 }
 
 // In place: S <- M^H(Re) - S (S holds R d on entry).
@@ -532,7 +533,7 @@ static int smooth32(const MixedCtx& C, int l, int sweeps, cudaStream_t st, bool 
           MG_DISPATCH32(C.m.kind, MG_CUDA_TRY(i32 ? go(k_smooth32s<KK, false, 0, int>) : go(k_smooth32s<KK>)));
           return MGGLAM_OK;
         }
-        const dim3 g((L.n / 4 + 31) / 32, L.n, (np + 3) / 4);
+        const dim3 g((L.n / 4 + 31) / 32, L.n / quad_rows(L.n), (np + 3) / 4);
         const bool i32 = L.n <= 1024;  // n^3 <= 2^30: 32-bit cell offsets
         if (wd && s == sweeps - 1) {
           MG_DISPATCH32(C.m.kind, (k_smooth32q<KK, true, int><<<g, dim3(32, 4), 0, st>>>(
@@ -598,7 +599,7 @@ static int fas_source(const MixedCtx& C, int l, cudaStream_t st) {
   Level& H = C.ws->lev[l];
   const float* rhoH = C.need_rho ? H.rho32 : nullptr;
   if (H.n % 4 == 0 && H.n >= 8) {
-    const dim3 g((H.n / 4 + 31) / 32, H.n, H.n / 4);
+    const dim3 g((H.n / 4 + 31) / 32, H.n / quad_rows(H.n), H.n / 4);
     if (H.n <= 1024) {  // 32-bit cell offsets
       MG_DISPATCH32(C.m.kind,
                     (k_fas_source32q<KK, int><<<g, dim3(32, 4), 0, st>>>(C.lf[l], H.n, H.Re, H.ub, rhoH, H.S32)));
@@ -854,7 +855,7 @@ static int restrict_level(const MixedCtx& C, int l, cudaStream_t st, bool relaxe
   Level& H = ws->lev[l + 1];
   const int bh = bx_for(H.n);
   if (l == 0 && C.split) {
-    const dim3 g((L.n / 4 + 31) / 32, H.n, (H.n + 3) / 4);
+    const dim3 g((L.n / 4 + 31) / 32, H.n / quad_rows(L.n), (H.n + 3) / 4);
     if (C.qs && relaxed) {
       // 32-bit cell offsets where the level has at most 2^30 cells
       auto kern = C.m.kind == KFR1 ? (L.n <= 1024 ? k_restrict32_split_zr<KFR1, int> : k_restrict32_split_zr<KFR1>)
@@ -878,7 +879,7 @@ static int restrict_level(const MixedCtx& C, int l, cudaStream_t st, bool relaxe
                                    C.lf[l], L.n, L.e, L.ub, rho, L.S32, H.Re, H.e, H.ub, H.S32, nullptr)));
     }
   } else if (L.n % 4 == 0 && L.n >= 8) {
-    const dim3 g((L.n / 4 + 31) / 32, H.n, (H.n + 3) / 4);
+    const dim3 g((L.n / 4 + 31) / 32, H.n / quad_rows(L.n), (H.n + 3) / 4);
     // 32-bit cell offsets where n^3 < 2^31
     if (relaxed && (C.m.kind != KCQ || cq_linear(C.lf[l]))) {
       if (L.n <= 1024) launch_restrict_quad<NatLayout32, true>(C, l, rho, g, st);
@@ -908,10 +909,10 @@ static int prolong_level(const MixedCtx& C, int l, cudaStream_t st, bool both = 
   Level& H = ws->lev[l + 1];
   const int bf = bx_for(L.n);
   if (l == 0 && C.split) {
-    const dim3 g((L.n / 4 + 31) / 32, L.n, L.n / 4);
+    const dim3 g((L.n / 4 + 31) / 32, L.n / quad_rows(L.n), L.n / 4);
     // with post-smoothing the first colour's corrections would be overwritten unread (prolong_quad)
     const bool second_only = !both && C.prm->nu2 >= 1 && second_colour_only(C);
-    const dim3 g2((L.n / 4 + 31) / 32, H.n, (H.n + 3) / 4);
+    const dim3 g2((L.n / 4 + 31) / 32, H.n / quad_rows(L.n), (H.n + 3) / 4);
     const bool dd = second_only && fine_reads_d(C);  // H.e_alt holds eH - Re
     const bool i32 = L.n <= 1024;  // 32-bit cell offsets
     if (C.qs && C.m.kind == KFR1 && dd)
@@ -940,7 +941,7 @@ static int prolong_level(const MixedCtx& C, int l, cudaStream_t st, bool both = 
       k_prolong_correct32q<true, SplitLayout><<<g, dim3(32, 4), 0, st>>>(H.n, H.e, H.Re, L.ub, L.e, C.guard);
     else k_prolong_correct32q<false, SplitLayout><<<g, dim3(32, 4), 0, st>>>(H.n, H.e, H.Re, L.ub, L.e, C.guard);
   } else if (L.n % 4 == 0 && L.n >= 8) {
-    const dim3 g((L.n / 4 + 31) / 32, L.n, L.n / 4);
+    const dim3 g((L.n / 4 + 31) / 32, L.n / quad_rows(L.n), L.n / 4);
     const bool i32 = L.n <= 1024;  // 32-bit cell offsets
     if (is_fr(C.m.kind) && i32)
       k_prolong_correct32q<true, NatLayout32><<<g, dim3(32, 4), 0, st>>>(H.n, H.e, H.Re, L.ub, L.e, C.guard);
