@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_setup(ModelDev m, int n, float
                                                         float* __restrict__ m32, float* __restrict__ dinv,
                                                         double* __restrict__ rhs, float* __restrict__ b,
                                                         double* __restrict__ partials) {
-  const double sl = K == KSYM ? m.msym * m.rat3 * ((double)n * n * n / *rho_sum) : 0.0;
+  const double sl = K == KSYM ? m.msym * m.rat3 * block_ratio((double)n * n * n, rho_sum) : 0.0;
   const double Kn = m.K / (K + 1), inp1 = 1.0 / (K + 1);
   const int h = n >> 1;
   const long long H = (long long)n * n * h;

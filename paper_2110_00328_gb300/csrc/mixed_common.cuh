@@ -547,7 +547,7 @@ static inline bool cq_linear(const LevelF& f) { return f.cq_series && fabsf(f.cq
 // CQ: the normalised density rho/mean in FP64 (the general residual's).
 static __global__ void k_src64(const float* __restrict__ rho32, long long n3, const double* __restrict__ rho_sum,
                                double* __restrict__ src) {
-  const double inv_mean = (double)n3 / *rho_sum;
+  const double inv_mean = block_ratio((double)n3, rho_sum);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x)
     src[t] = inv_mean * (double)rho32[t];
@@ -1139,7 +1139,7 @@ __global__ void __launch_bounds__(TJ* TK) k_cq_residual(ModelDev m, CqSeries q, 
 // rho32 normalised to mean 1 (FP64 mean), for the inner levels.
 static __global__ void k_density_norm32(const float* __restrict__ rho, long long n3, const double* __restrict__ sum,
                                  float* __restrict__ out) {
-  const float im = (float)((double)n3 / *sum);
+  const float im = (float)block_ratio((double)n3, sum);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x)
     out[t] = rho[t] * im;
@@ -1149,7 +1149,7 @@ static __global__ void k_density_norm32(const float* __restrict__ rho, long long
 static __global__ void k_density_norm32_split(const float* __restrict__ rho, int n, const double* __restrict__ sum,
                                               float* __restrict__ out) {
   const long long n3 = (long long)n * n * n;
-  const float im = (float)((double)n3 / *sum);
+  const float im = (float)block_ratio((double)n3, sum);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(t % n), j = (int)((t / n) % n), i = (int)(t / ((long long)n * n));
@@ -1190,7 +1190,7 @@ static __global__ void k_src_sumsq32(ModelDev m, const float* __restrict__ rho32
   // a normalisation scale: single precision per cell is ample.  delta =
   // rho/mean - 1 is formed with an FMA against the two-float 1/mean, so it
   // keeps its relative precision where rho is close to the mean.
-  const double inv_mean = (double)n3 / *rho_sum;
+  const double inv_mean = block_ratio((double)n3, rho_sum);
   const float im_hi = (float)inv_mean, im_lo = (float)(inv_mean - (double)im_hi);
   float acc = 0.f;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
@@ -1203,8 +1203,10 @@ static __global__ void k_src_sumsq32(ModelDev m, const float* __restrict__ rho32
   if constexpr (is_fr(K)) f = m.om_a;
   else if constexpr (K == KSYM) f = m.msym * m.rat3 * m.ubar;
   else f = m.cq_src;
-  const double a = block_sum((double)acc * (f * f));
-  if (threadIdx.x == 0) partials[blockIdx.x] = a;
+  FloatFloat v;
+  v.hi = acc;
+  const double a = block_sum(v);
+  if (threadIdx.x == 0) partials[blockIdx.x] = a * (f * f);
 }
 
 static __global__ void k_finalize_sum32(const double* __restrict__ partials, int count, double* __restrict__ out) {

@@ -245,14 +245,14 @@ __global__ void k_sum_f32(const float* __restrict__ x, long long n3, double* __r
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x)
     acc.add(x[t]);
-  const double a = block_sum(acc.value());
+  const double a = block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = a;
 }
 
 // rho64 = rho32 / mean, mean = sum / n3 read from device memory.
 __global__ void k_density_to64(const float* __restrict__ rho32, long long n3, const double* __restrict__ sum,
                                double* __restrict__ rho64) {
-  const double inv_mean = (double)n3 / *sum;
+  const double inv_mean = block_ratio((double)n3, sum);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x)
     rho64[t] = (double)rho32[t] * inv_mean;
