@@ -390,8 +390,8 @@ double mgglam_radiation_density(double h);
  *   N    power of two, 8 <= N <= 1024.
  *   coef for the Newtonian potential (3/2) Om / a.
  *   phi  device, N^3 float32 output (may not alias rho).
- * The library keeps an N^3 complex work array per (device, N), freed by
- * mgglam_release.  Errors: MGGLAM_ERR_ARG, MGGLAM_ERR_SHAPE, MGGLAM_ERR_OOM,
+ * The library keeps a work array of the N x N x (N/2 + 1) complex modes (rows padded to
+ * 128 bytes) per (device, N), freed by mgglam_release.  Errors: MGGLAM_ERR_ARG, MGGLAM_ERR_SHAPE, MGGLAM_ERR_OOM,
  * MGGLAM_ERR_CUDA.
  */
 int mgglam_poisson_fft(const float* rho, int N, double coef, float* phi, void* stream);
