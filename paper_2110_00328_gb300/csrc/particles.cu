@@ -13,11 +13,11 @@
 // difference (T_{c+1} - T_{c-1})/2 free of cancellation in single precision.
 // Each particle then interpolates the three-point differences of the 8 cells
 // around it with its CIC weights.
-#include <cuda_pipeline.h>
 #include <math.h>
 
 #include <mutex>
 
+#include "bricks.cuh"
 #include "cic.cuh"
 #include "ff.cuh"
 #include "mg_common.cuh"
@@ -80,7 +80,9 @@ __device__ __forceinline__ unsigned long long wmul29(unsigned long long P, unsig
 // does not depend on which lane issues an update.
 template <typename IT>
 __global__ void __launch_bounds__(kThreads) k_deposit_fixed(const float* __restrict__ pos, long long np, int N,
-                                                            unsigned long long* __restrict__ acc) {
+                                                            unsigned long long* __restrict__ acc,
+                                                            const int* by_bricks) {
+  if (by_bricks && *by_bricks) return;
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < np; base += stride) {
@@ -143,11 +145,10 @@ __global__ void __launch_bounds__(kThreads) k_deposit_fixed(const float* __restr
 // 2048 weights of at most 2^32 fit.  A particle outside the window (1% of 256^3
 // Zel'dovich particles of pixel sigma 1.5) goes to the mesh directly, so any
 // positions are taken; the integer sums are the same in any order.
-// Measured (those particles, the whole call): 470 us before, 325 now; 160^3 cells,
-// 200^3 particles 208 and 158.  Issue slots (69%) and the 16 shared atomics a
+// Measured (those particles, the whole call): 470 us before, 325 by this kernel alone, 343
+// with k_brick_probe and the other kernel's launch; pixel sigma 5: 652 and 474.  Issue slots (69%) and the 16 shared atomics a
 // particle (L1 68%) share the bound; 32-bit sums with a carry (8 atomics and few
 // carries a particle) are no faster, nor are two CTAs an SM (348).
-constexpr int kBrickI = 8, kBrickJ = 8, kBrickK = 32;            // particles
 constexpr int kWinI = 14, kWinJ = 14, kWinK = 40;               // cells
 constexpr int kWinCells = kWinI * kWinJ * kWinK;
 constexpr int kBrickThreads = 512, kBrickPer = kBrickI * kBrickJ * kBrickK / kBrickThreads;
@@ -175,7 +176,9 @@ __device__ __noinline__ void deposit_direct(const float* __restrict__ x, int N, 
 template <typename IT>
 __global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float* __restrict__ pos, int M, int ni,
                                                                      int nbj, int nbk, int N,
-                                                                     unsigned long long* __restrict__ acc) {
+                                                                     unsigned long long* __restrict__ acc,
+                                                                     const int* by_bricks) {
+  if (!*by_bricks) return;
   extern __shared__ unsigned win[];  // low words, then high words
   __shared__ int s_sum[4], s_nout;
   __shared__ unsigned short s_out[kBrickOut];  // particles outside the window
@@ -276,36 +279,31 @@ __global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float
   }
 }
 
-// The deposit of np particles on acc: of an M x M x ... array (M^2 a divisor of np) of
-// at least two bricks an SM and half a particle a cell -- below that the window's
-// zeroing and flush, four cells a particle, cost more than the atomics they save --
-// in a mesh of at least the window's longest side brick by brick, else in the order
-// of the array.  lattice: M, or 0.
+// The deposit of np particles on acc, brick by brick (brick_grid; at fewer particles the
+// window's zeroing and flush, four cells a particle, cost more than the atomics they
+// save) or in the order of the array.  lattice: M, or 0.  The word behind acc's N^3 says
+// which of the two (k_brick_probe).
 static int launch_deposit(const float* pos, long long np, long long lattice, int N, unsigned long long* acc,
                           cudaStream_t st) {
-  const long long M = lattice, ni = M > 0 ? np / (M * M) : 0;
-  const long long nbj = (M + kBrickJ - 1) / kBrickJ, nbk = (M + kBrickK - 1) / kBrickK,
-                  blocks = (ni + kBrickI - 1) / kBrickI * nbj * nbk;
-  if (M > 0 && M <= 65536 && N >= kWinK && ni * M * M == np && 2 * M * M * M >= (long long)N * N * N && blocks >= 304 &&
-      blocks <= 0x7fffffffLL) {
+  const BrickGrid b = brick_grid(np, lattice, N, kWinK);
+  if (b.blocks) {
     constexpr int smem = 2 * kWinCells * (int)sizeof(unsigned);
     auto kern = N <= 1024 ? k_deposit_bricks<int> : k_deposit_bricks<long long>;
     MG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<(unsigned)blocks, kBrickThreads, smem, st>>>(pos, (int)M, (int)ni, (int)nbj, (int)nbk, N, acc);
+    int* by_bricks = reinterpret_cast<int*>(acc + (long long)N * N * N);
+    k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
+    kern<<<b.blocks, kBrickThreads, smem, st>>>(pos, b.M, b.ni, b.nbj, b.nbk, N, acc, by_bricks);
+    (N <= 1024 ? k_deposit_fixed<int> : k_deposit_fixed<long long>)<<<grid_for(np, kThreads, kBrickOther), kThreads, 0,
+                                                                       st>>>(pos, np, N, acc, by_bricks);
+    note_launch(2);
   } else {
     // 32-bit cell offsets where the mesh has at most 2^30 cells
     (N <= 1024 ? k_deposit_fixed<int> : k_deposit_fixed<long long>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0,
-                                                                       st>>>(pos, np, N, acc);
+                                                                       st>>>(pos, np, N, acc, nullptr);
   }
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
-}
-
-// The side M of an array of M^3 particles, or 0.
-static long long lattice_side(long long np) {
-  const long long M = llround(cbrt((double)np));
-  return M * M * M == np ? M : 0;
 }
 
 __global__ void k_deposit_finish(const unsigned long long* __restrict__ acc, long long n3, double mass,
@@ -323,7 +321,7 @@ static int deposit_scratch(int N, unsigned long long** acc) {
   Workspace* ws = nullptr;
   int rc = get_workspace(N < 4 ? 4 : (N % 2 ? N + 1 : N), MGGLAM_FP64, 1, &ws);
   if (rc) return rc;
-  const size_t need = (size_t)N * N * N * sizeof(unsigned long long);
+  const size_t need = ((size_t)N * N * N + 1) * sizeof(unsigned long long);  // and by_bricks
   if (ws->cic_bytes < need) {
     if (ws->cic_acc) cudaFree(ws->cic_acc);
     ws->cic_acc = nullptr;
@@ -388,7 +386,9 @@ __global__ void k_transform(const double* __restrict__ u, long long n3, double u
 // differences at the 8 CIC cells touch).
 template <typename IT>
 __global__ void __launch_bounds__(kThreads) k_gather(const float* __restrict__ T, int N, const float* __restrict__ pos,
-                                                     long long np, float scale, float* __restrict__ force) {
+                                                     long long np, float scale, float* __restrict__ force,
+                                                     const int* by_bricks) {
+  if (by_bricks && *by_bricks) return;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < np;
        q += (long long)gridDim.x * blockDim.x) {
     const float3 g = cic_grad<IT>(T, N, pos[3 * q + 0], pos[3 * q + 1], pos[3 * q + 2]);
@@ -398,161 +398,42 @@ __global__ void __launch_bounds__(kThreads) k_gather(const float* __restrict__ T
   }
 }
 
-// The same gather for lattice-ordered particles, brick by brick.
-//
-// k_gather is bound by L1: its 32 loads a particle hit about seven lines a warp
-// (320 us at 256^3).  As in k_deposit_bricks a CTA takes a brick of 8 x 8 x 32 of the
-// array and stages the window of the mesh about the brick's mean displacement in
-// shared memory, whose banks serve the scattered lanes side by side.  The window's
-// rows start at multiples of four cells, so that they arrive as 16-byte copies (four
-// times fewer instructions) where N is one too.  A particle outside the window reads
-// the mesh itself, after the others.  The sums are cic_grad's, in its order.
-// Measured (256^3 Zel'dovich particles of pixel sigma 1.5, with the transform's 39 us):
-// 359 us before, 270 now (sigma 2.5: 518 and 333); 160^3 cells, 200^3 particles 170 and
-// 131; 314^3 cells, 253^3 particles 441 and 388.  More warps matter more than a wider
-// window: 16 x 16 x 48 cells 274 us, three CTAs an SM 302, 512 threads a CTA 310.
-constexpr int kTileI = 15, kTileJ = 15, kTileK = 48;  // cells
-constexpr int kTileCells = kTileI * kTileJ * kTileK;
-constexpr int kTilePlanes = 1;                        // of a brick at a time
-constexpr int kTileThreads = kTilePlanes * kBrickJ * kBrickK;
-constexpr int kTileOut = 512;
-
-template <typename IT>
-__device__ __noinline__ void gather_direct(const float* __restrict__ T, int N, const float* __restrict__ x, float scale,
-                                           float* __restrict__ out) {
-  const float3 g = cic_grad<IT>(T, N, x[0], x[1], x[2]);
-  out[0] = scale * g.x;
-  out[1] = scale * g.y;
-  out[2] = scale * g.z;
-}
-
+// The same gather brick by brick (brick_gradients).  Measured (256^3 Zel'dovich
+// particles of pixel sigma 1.5, with the transform's 39 us): 359 us before, 270 by this
+// kernel alone, 289 with k_brick_probe and the other kernel's launch; sigma 3: 604 and 387.
 template <typename IT, bool QUADS>
 __global__ void __launch_bounds__(kTileThreads, 4) k_gather_bricks(const float* __restrict__ T, int N,
-                                                                   const float* __restrict__ pos, int M, int ni,
-                                                                   int nbj, int nbk, float scale,
-                                                                   float* __restrict__ force) {
-  extern __shared__ __align__(16) float tile[];
-  __shared__ int s_sum[4], s_nout;
-  __shared__ unsigned short s_out[kTileOut];  // particles outside the window
-  const int t = threadIdx.x;
-  const unsigned b = blockIdx.x, bij = b / (unsigned)nbk, bk = b - bij * nbk, bi = bij / (unsigned)nbj,
-                 bj = bij - bi * nbj;
-  const int i0 = bi * kBrickI + t / (kBrickJ * kBrickK), j0 = bj * kBrickJ + (t / kBrickK) % kBrickJ,
-            k0 = bk * kBrickK + t % kBrickK;
-  const long long brick = ((long long)bi * kBrickI * M + bj * kBrickJ) * M + bk * kBrickK;  // its first particle
-  const long long mine = ((long long)i0 * M + j0) * M + k0;                                 // this thread's first
-  const long long plane = (long long)kTilePlanes * M * M;                                   // and the next ones' distance
-  const int mp = j0 < M && k0 < M && i0 < ni
-                     ? min(kBrickI / kTilePlanes, (ni - i0 + kTilePlanes - 1) / kTilePlanes)
-                     : 0;  // this thread's particles
-  if (t < 4) s_sum[t] = 0;
-  if (t == 4) s_nout = 0;
-  __syncthreads();
-  // window origin: the mean place of a middle plane's particles, measured from the brick's first one, less half a window
-  const float ref[3] = {wrap_pos(pos[3 * brick], N), wrap_pos(pos[3 * brick + 1], N), wrap_pos(pos[3 * brick + 2], N)};
-  {
-    const float fN = (float)N, iN = 1.f / (float)N;
-    int sum[4] = {0, 0, 0, mp > 0};
-    if (mp > 0) {
-      const float* x = pos + 3 * (mine + (mp >> 1) * plane);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const float o = x[d] - ref[d];
-        sum[d] = (int)rintf(o - fN * rintf(o * iN));  // nearest image
-      }
-    }
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      const int w = __reduce_add_sync(0xffffffffu, sum[d]);
-      if ((t & 31) == 0) atomicAdd(&s_sum[d], w);
-    }
-  }
-  __syncthreads();
-  int org[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int half = (d == 0 ? kTileI : (d == 1 ? kTileJ : kTileK)) / 2;
-    org[d] = ((int)(ref[d] + __fdividef((float)s_sum[d], (float)s_sum[3])) - half) % N;
-    org[d] += org[d] < 0 ? N : 0;
-  }
-  if (QUADS) {
-    org[2] &= ~3;
-#pragma unroll 4
-    for (int a = t; a < kTileCells / 4; a += kTileThreads) {
-      const int ij = a / (kTileK / 4), wi = ij / kTileJ;
-      int i = org[0] + wi, j = org[1] + ij - wi * kTileJ, k = org[2] + 4 * (a - ij * (kTileK / 4));
-      i -= i >= N ? N : 0;  // N >= the window's sides: one wrap
-      j -= j >= N ? N : 0;
-      k -= k >= N ? N : 0;
-      __pipeline_memcpy_async(tile + 4 * a, T + ((IT)i * N + j) * N + k, 16);
-    }
-    __pipeline_commit();
-    __pipeline_wait_prior(0);
-  } else {
-#pragma unroll 4
-    for (int a = t; a < kTileCells; a += kTileThreads) {
-      const int ij = a / kTileK, wi = ij / kTileJ;
-      int i = org[0] + wi, j = org[1] + ij - wi * kTileJ, k = org[2] + a - ij * kTileK;
-      i -= i >= N ? N : 0;
-      j -= j >= N ? N : 0;
-      k -= k >= N ? N : 0;
-      tile[a] = T[((IT)i * N + j) * N + k];
-    }
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int r = 0; r < mp; ++r) {
-    const long long p = 3 * (mine + r * plane);
-    int c[3], c1;
-    float w[3][2];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      cic_axis_f(pos[p + d], N, c[d], c1, w[d][0], w[d][1]);
-      c[d] -= org[d];
-      c[d] += c[d] < 0 ? N : 0;
-    }
-    if (c[0] >= 1 && c[0] + 2 < kTileI && c[1] >= 1 && c[1] + 2 < kTileJ && c[2] >= 1 && c[2] + 2 < kTileK) {
-      const float* at = tile + ((c[0] - 1) * kTileJ + c[1] - 1) * kTileK + c[2] - 1;
-      const float3 g =
-          cic_grad_core([&](int a, int bb, int cc) { return at[(a * kTileJ + bb) * kTileK + cc]; }, w[0], w[1], w[2]);
-      force[p] = scale * g.x;
-      force[p + 1] = scale * g.y;
-      force[p + 2] = scale * g.z;
-    } else {
-      const int q = atomicAdd(&s_nout, 1);
-      if (q < kTileOut) s_out[q] = (unsigned short)(t + r * kTileThreads);
-      else gather_direct<IT>(T, N, pos + p, scale, force + p);
-    }
-  }
-  __syncthreads();
-  for (int q = t; q < min(s_nout, kTileOut); q += kTileThreads) {
-    const int x = s_out[q];
-    const int i = x / (kBrickJ * kBrickK), j = (x / kBrickK) % kBrickJ, k = x % kBrickK;
-    const long long p = 3 * (brick + ((long long)i * M + j) * M + k);
-    gather_direct<IT>(T, N, pos + p, scale, force + p);
-  }
+                                                                   const float* __restrict__ pos, BrickGrid b,
+                                                                   float scale, float* __restrict__ force,
+                                                                   const int* by_bricks) {
+  if (!*by_bricks) return;
+  brick_gradients<IT, QUADS>(T, N, pos, b, [&](long long p, const float*, float3 g) {
+    force[p] = scale * g.x;
+    force[p + 1] = scale * g.y;
+    force[p + 2] = scale * g.z;
+  });
 }
 
-// The gather of np particles: brick by brick where the deposit would be (at the rule's
-// edge, two cells a particle, 388 us against 441), in a mesh of at least the window's
-// longest side.  lattice: as launch_deposit's.
+// The gather of np particles: brick by brick where the deposit would be, in a mesh of at
+// least the window's longest side.  lattice: as launch_deposit's.
 static int launch_gather(const float* T, int N, const float* pos, long long np, long long lattice, float scale,
-                         float* force, cudaStream_t st) {
-  const long long M = lattice, ni = M > 0 ? np / (M * M) : 0;
-  const long long nbj = (M + kBrickJ - 1) / kBrickJ, nbk = (M + kBrickK - 1) / kBrickK,
-                  blocks = (ni + kBrickI - 1) / kBrickI * nbj * nbk;
-  if (M > 0 && M <= 65536 && N >= kTileK && ni * M * M == np && 2 * M * M * M >= (long long)N * N * N && blocks >= 304 &&
-      blocks <= 0x7fffffffLL) {
+                         float* force, int* by_bricks, cudaStream_t st) {
+  const BrickGrid b = brick_grid(np, lattice, N, kTileK);
+  if (b.blocks) {
     constexpr int smem = kTileCells * (int)sizeof(float);
     const bool quads = N % 4 == 0;  // T's rows on 16-byte boundaries (the workspace's mesh is)
     auto kern = N <= 1024 ? (quads ? k_gather_bricks<int, true> : k_gather_bricks<int, false>)
                           : (quads ? k_gather_bricks<long long, true> : k_gather_bricks<long long, false>);
     MG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<(unsigned)blocks, kTileThreads, smem, st>>>(T, N, pos, (int)M, (int)ni, (int)nbj, (int)nbk, scale, force);
+    k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
+    kern<<<b.blocks, kTileThreads, smem, st>>>(T, N, pos, b, scale, force, by_bricks);
+    (N <= 1024 ? k_gather<int> : k_gather<long long>)<<<grid_for(np, kThreads, kBrickOther), kThreads, 0, st>>>(
+        T, N, pos, np, scale, force, by_bricks);
+    note_launch(2);
   } else {
     // 32-bit cell offsets where the mesh has at most 2^30 cells
     (N <= 1024 ? k_gather<int> : k_gather<long long>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0, st>>>(
-        T, N, pos, np, scale, force);
+        T, N, pos, np, scale, force, nullptr);
   }
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
@@ -577,7 +458,8 @@ int gather_chunk(const ModelDev& m, int kind, const mgglam_params* prm, int N, c
   if (rc) return rc;
   const float* T = ws->lev[0].ub;
   prof_begin(PC_GATHER, st, 24.0 * np);
-  rc = launch_gather(T, N, pos, np, lattice, (float)(force_scale(m, kind, prm) * prefactor), force, st);
+  rc = launch_gather(T, N, pos, np, lattice, (float)(force_scale(m, kind, prm) * prefactor), force,
+                     by_bricks_of(ws), st);
   prof_end(st);
   return rc;
 }
@@ -604,7 +486,8 @@ int gather_force(const ModelDev& m, int kind, int n_fr, const mgglam_params* prm
   scale = force_scale(m, kind, prm);
   prof_begin(PC_GATHER, st, 24.0 * np + 4.0 * n3);
   note_launch(1);
-  rc = launch_gather(T, N, pos, np, lattice < 0 ? lattice_side(np) : lattice, (float)(scale * prefactor), force, st);
+  rc = launch_gather(T, N, pos, np, lattice < 0 ? lattice_side(np) : lattice, (float)(scale * prefactor), force,
+                     by_bricks_of(ws), st);
   prof_end(st);
   return rc;
 }
@@ -731,7 +614,7 @@ constexpr int kStaticDepositMaxN = 128;
 constexpr size_t kStaticDepositCells = (size_t)kStaticDepositMaxN * kStaticDepositMaxN * kStaticDepositMaxN;
 constexpr int kStaticMaxDevices = 64;
 
-static __device__ __align__(256) unsigned long long g_static_deposit_acc[kStaticDepositCells];
+static __device__ __align__(256) unsigned long long g_static_deposit_acc[kStaticDepositCells + 1];  // and by_bricks
 
 static std::mutex g_static_mu;
 static unsigned long long* g_static_acc_ptr[kStaticMaxDevices];

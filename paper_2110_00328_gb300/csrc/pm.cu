@@ -76,6 +76,7 @@ __device__ __forceinline__ float cic_interp64(const double* __restrict__ u, int 
 // Kick and drift of every particle.  kick = da H0/adot(a_n); drift = da H0/(a^2 adot) at
 // a_n + da/2; gdrag = gamma da for a uniform drag (CQ); sym_drag = the symmetron's
 // gamma da per unit u (0 when absent), u interpolated from the field.
+template <typename IT>  // the index type of the cell offsets
 __global__ void __launch_bounds__(kThreads) k_pm_kick_drift(const float* __restrict__ psi, int N,
                                                             float* __restrict__ pos, float* __restrict__ mom,
                                                             long long np, float kick, float drift, float gdrag,
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(kThreads) k_pm_kick_drift(const float* __restr
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < np;
        q += (long long)gridDim.x * blockDim.x) {
     const float x = pos[3 * q + 0], y = pos[3 * q + 1], z = pos[3 * q + 2];
-    const float3 g = cic_grad(psi, N, x, y, z);
+    const float3 g = cic_grad<IT>(psi, N, x, y, z);
     float gd = gdrag;
     if (sym_drag != 0.f) gd += sym_drag * cic_interp64(field, N, x, y, z);
     const float c0 = 1.f - 0.5f * gd, ci = 1.f / (1.f + 0.5f * gd);
@@ -155,8 +156,9 @@ int pm_step(const mgglam_params* prm, const mgglam_pm_step_desc* d, int N, float
                        sqrt(1.0 - r * r * r) / (a * a * a * a) * da);
   }
   prof_begin(PC_PM_KICK_DRIFT, st, 48.0 * np + 4.0 * n3);
-  k_pm_kick_drift<<<grid_for(np, kThreads, 1 << 20), kThreads, 0, st>>>(psi_work, N, pos, mom, np, kick, drift,
-                                                                         gdrag, sym_drag, field);
+  // 32-bit cell offsets where the mesh has at most 2^30 cells
+  (N <= 1024 ? k_pm_kick_drift<int> : k_pm_kick_drift<long long>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0, st>>>(
+      psi_work, N, pos, mom, np, kick, drift, gdrag, sym_drag, field);
   prof_end(st);
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());

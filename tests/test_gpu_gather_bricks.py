@@ -19,7 +19,7 @@ torch = pytest.importorskip("torch")
 # mesh sides below, at and above the window's, multiples of four (16-byte rows) and not;
 # M with whole and partial bricks
 @pytest.mark.parametrize("N", [30, 48, 50, 64, 98, 120])
-@pytest.mark.parametrize("M", [96, 101])
+@pytest.mark.parametrize("M", [185, 192])
 @pytest.mark.parametrize("kind", ["lattice", "random", "clump", "two clumps", "wrap"])
 def test_bricks_equal_singles(mg, N, M, kind):  # noqa: F811
     rng = np.random.default_rng(M + N)
