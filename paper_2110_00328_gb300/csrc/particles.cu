@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float
                                                                      unsigned long long* __restrict__ acc,
                                                                      const int* by_bricks) {
   if (!*by_bricks) return;
-  extern __shared__ unsigned win[];  // low words, then high words
+  extern __shared__ __align__(16) unsigned win[];  // low words, then high words; cleared 16 bytes at a time
   __shared__ int s_sum[4], s_nout;
   __shared__ unsigned short s_out[kBrickOut];  // particles outside the window
   const int t = threadIdx.x;
