@@ -27,6 +27,7 @@
 #include <chrono>
 #include <mutex>
 
+#include "adjoint_levels.h"
 #include "ff.cuh"
 #include "fp64_fast.cuh"
 #include "mg_common.cuh"
@@ -493,7 +494,7 @@ __global__ void __launch_bounds__(128) k_adj_prolong_split(int nc, const float* 
 // and eight operations, so even a 16^3 colour pass is shorter there than a
 // kernel's start.  A level's x starts at zero, the finest mesh's (warm) from
 // where the cycle before left it.
-constexpr int kAdjTailCells = 4096, kAdjTailThreads = 1024, kAdjTailLevels = 5;
+constexpr int kAdjTailThreads = 1024;
 struct AdjTail {
   int T;                     // levels
   int n[kAdjTailLevels];
@@ -505,12 +506,6 @@ struct AdjTail {
   int nu1, nu2, sweeps;
   int warm;                  // the first level's x is read
 };
-
-static inline size_t adj_tail_smem(const AdjTail& A) {
-  size_t cells = 0;
-  for (int l = 0; l < A.T; ++l) cells += (size_t)A.n[l] * A.n[l] * A.n[l];
-  return cells * 4 * sizeof(float);
-}
 
 __device__ __forceinline__ float adj_tail_sum(const float* x, int n, int i, int j, int k) {
   const int nn = n * n, c = (i * n + j) * n + k;
@@ -973,7 +968,7 @@ static int adj_vcycle(const AdjCtx& C, int l, bool fresh, cudaStream_t st) {
     A.nu2 = prm->nu2;
     A.sweeps = prm->coarse_sweeps;
     A.warm = !fresh;
-    k_adj_tail<<<1, kAdjTailThreads, adj_tail_smem(A), st>>>(A);
+    k_adj_tail<<<1, kAdjTailThreads, adj_tail_smem(A.n, A.T), st>>>(A);
     note_launch(1);
     return MGGLAM_OK;
   }
@@ -1027,10 +1022,9 @@ int solve_adjoint(const mgglam_params* prm, double a, const double* field, const
   const long long n3 = (long long)N * N * N;
   if ((rc = launch_density_mean(rho, (size_t)n3, ws->partials, ws->scalars + SC_MEAN, st))) return rc;
   AdjCtx C = {w, prm, m.c2, N % 32 == 0 && prm->nu1 >= 1 && prm->nu2 >= 1, -1};
-  for (int l = 0; l < w->nlev && C.tail < 0; ++l)
-    if ((l > 0 || !C.split) && w->nlev - l <= kAdjTailLevels && w->n[l] * w->n[l] * w->n[l] <= kAdjTailCells) C.tail = l;
-  if (C.tail >= 0)  // at most 4 arrays of 4096 (1 + 1/8 + ...) cells
-    MG_CUDA_TRY(cudaFuncSetAttribute(k_adj_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024));
+  C.tail = adj_tail_level(w->n, w->nlev, C.split);
+  if (C.tail >= 0)
+    MG_CUDA_TRY(cudaFuncSetAttribute(k_adj_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjTailSmem));
   const int rows = N * N < kMaxReduceBlocks ? N * N : kMaxReduceBlocks;  // grid of the row kernels
   const int bh = N >= 512 ? 256 : (N <= 64 ? 32 : ((N / 2 + 31) / 32) * 32);  // their threads, one per pair of cells
   const double* rs = ws->scalars + SC_MEAN;
