@@ -15,12 +15,14 @@
 // mesh, each one read and one write:
 //   z forward (real density in) -> y forward -> x forward, times the Green's
 //   function, x inverse (one kernel) -> y inverse -> z inverse (real Phi out).
+// A sixth launch, behind the first, transforms a density far from unit mean again,
+// times a power of two.
 // The density is real, so a z row is transformed as M = N/2 complex values
 // x[2m] + i x[2m+1] and only its M + 1 independent modes are kept: every pass
 // moves half of what complex rows move (40 instead of 72 bytes a cell), and at
 // 256^3 the 67 MB of modes stay in the 126 MB L2 between passes while the density
-// and the potential stream past them.  Measured with the density's sum: 149 us at
-// 256^3 (257 us with complex rows), 1.56 ms at 512^3 (2.65); the row passes take
+// and the potential stream past them.  Measured with the density's sum: 143 us at
+// 256^3 (257 us with complex rows), 1.58 ms at 512^3 (2.65); the row passes take
 // about 35 and 42 us of it, bound by shared-memory and instruction issue between
 // their barriers, the column passes 24, 34 and 24 us.
 // z is the contiguous axis: a CTA transforms whole rows.  For y and x a CTA
@@ -148,6 +150,27 @@ __device__ __forceinline__ ff warp_sum_ff(ff v) {
   return v;
 }
 
+// Every pass but the first is a programmatic dependent launch (launch_pass): its CTAs
+// are set up while the previous pass drains, and wait for its end here.
+__device__ __forceinline__ void after_previous_pass() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// What the passes after the forward rows take of the density's mean.
+struct FftScale {
+  float green;   // -coef over the mean of what was transformed
+  float factor;  // the rows are to be transformed again, times this power of two; 0: no
+};
+
+// The factor of the second transform.  The sums of a density in units of its own
+// must stay within float's range -- up to 2 N^3 <= 2^31 times the mean, and the
+// small modes above the subnormals -- and so must -coef / mean.  Means within 2^20
+// of 1 leave room for all of them; the others are brought near 1, exactly.
+__device__ __forceinline__ float fft_factor(double mean, double green) {
+  const double m = fabs(mean), g = fabs(green);
+  if (!(m < INFINITY)) return 0x1p-100f;  // the sum overflowed (or the density holds an infinity or a NaN)
+  if (m == 0.0 || g == 0.0 || (m >= 0x1p-20 && m <= 0x1p20 && g >= 0x1p-100 && g <= 0x1p100)) return 0.f;
+  return ldexpf(1.f, max(-126, min(-ilogb(m), 127)));
+}
+
 // Contiguous axis (z) forward, L whole rows of N = 2M reals per CTA, M = R1 R2.
 // Each phase deals its own work to the CTA's threads, so that whole warps are
 // either busy or done: L R2 threads load z[R2 n1 + r], z[m] = x[2m] + i x[2m+1],
@@ -158,77 +181,99 @@ __device__ __forceinline__ ff warp_sum_ff(ff v) {
 //   2 X[k] = E + W_N^k O,  2 X[M-k] = conj(E - W_N^k O)
 // (the factor 2 goes into the inverse's scale).
 // The pass also sums the density (float-float per CTA; the last CTA to finish adds
-// the partial sums in order) and leaves N^3 / sum, which the Green's function
-// takes in: a separate pass over the density took 28 us at 256^3.  pairs: rho is
-// 8-byte aligned.
-template <int R1, int R2>
+// the partial sums in order) and leaves -coef over its mean, which the Green's
+// function takes in: a separate pass over the density took 28 us at 256^3.
+// AGAIN: the pass over a density whose mean the first one found far from 1
+// (fft_factor), a grid-stride loop whose CTAs otherwise return at once (4 us as an
+// ordinary launch; with the dependent launches the whole call takes 143 us at 256^3,
+// 150 without either, and 173 for a density of mean 1e35).
+// pairs: rho is 8-byte aligned.
+template <int R1, int R2, bool AGAIN>
 __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_rfft_rows_fwd(
-    const float* __restrict__ rho, float2* __restrict__ modes, bool pairs, const float2* __restrict__ twN,
-    const float2* __restrict__ twM, double* __restrict__ partials, unsigned* __restrict__ ticket,
-    float* __restrict__ inv_mean) {
-  constexpr int M = R1 * R2, N = 2 * M, S = mode_stride(N), L = rows_per_cta(N), NT = L * R2;
+    const float* __restrict__ rho, float2* __restrict__ modes, bool pairs, double coef,
+    const float2* __restrict__ twN, const float2* __restrict__ twM, double* __restrict__ partials,
+    unsigned* __restrict__ ticket, FftScale* scale) {
+  constexpr int M = R1 * R2, N = 2 * M, S = mode_stride(N), L = rows_per_cta(N), NT = L * R2, H = M / 2;
   static_assert(R2 >= R1, "one thread per load of the first phase");
   extern __shared__ float2 fft_sm[];
   __shared__ ff s_part[kFftThreads / 32];
   __shared__ bool s_last;
   const int t = threadIdx.x;
-  const long long row0 = (long long)blockIdx.x * L;
+  if (AGAIN) after_previous_pass();
+  const float factor = AGAIN ? scale->factor : 1.f;
+  if (AGAIN && factor == 0.f) return;
   float2* Zs = fft_sm + L * row_ex<R1, R2>();
   FloatFloat acc;
-  {
-    const int l = t / R2, r = t - l * R2;
-    const float* x = rho + 2 * ((row0 + l) * M + r);
-    float2 v[R1];
-    if (pairs) {
+  auto rows = [&](unsigned block) {
+    const long long row0 = (long long)block * L;
+    {
+      const int l = t / R2, r = t - l * R2;
+      const float* x = rho + 2 * ((row0 + l) * M + r);
+      float2 v[R1];
+      if (pairs) {
 #pragma unroll
-      for (int n1 = 0; n1 < R1; ++n1) v[n1] = __ldcs(reinterpret_cast<const float2*>(x + 2 * R2 * n1));
-    } else {
+        for (int n1 = 0; n1 < R1; ++n1) v[n1] = __ldcs(reinterpret_cast<const float2*>(x + 2 * R2 * n1));
+      } else {
 #pragma unroll
-      for (int n1 = 0; n1 < R1; ++n1) v[n1] = make_float2(x[2 * R2 * n1], x[2 * R2 * n1 + 1]);
+        for (int n1 = 0; n1 < R1; ++n1) v[n1] = make_float2(x[2 * R2 * n1], x[2 * R2 * n1 + 1]);
+      }
+#pragma unroll
+      for (int n1 = 0; n1 < R1; ++n1) {
+        if (AGAIN) v[n1] = make_float2(v[n1].x * factor, v[n1].y * factor);
+        acc.add(v[n1].x);
+        acc.add(v[n1].y);
+      }
+      float2* Y = fft_sm + l * row_ex<R1, R2>() + r;
+      fft_phase1<R1, R2, false, true>(v, r, twM, [&](int k1) -> float2& { return Y[k1 * (R2 + 1)]; });
     }
-#pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1) {
-      acc.add(v[n1].x);
-      acc.add(v[n1].y);
+    if (!AGAIN) {
+      const ff w = warp_sum_ff(ff{acc.hi, acc.lo});
+      if ((t & 31) == 0) s_part[t >> 5] = w;
     }
-    float2* Y = fft_sm + l * row_ex<R1, R2>() + r;
-    fft_phase1<R1, R2, false, true>(v, r, twM, [&](int k1) -> float2& { return Y[k1 * (R2 + 1)]; });
-  }
-  const ff w = warp_sum_ff(ff{acc.hi, acc.lo});
-  if ((t & 31) == 0) s_part[t >> 5] = w;
-  __syncthreads();
-  if (t < L * R1) {
-    const int l = t / R1, r = t - l * R1;
-    const float2* Y = fft_sm + l * row_ex<R1, R2>() + r * (R2 + 1);
-    float2 u[R2];
+    __syncthreads();
+    if (t < L * R1) {
+      const int l = t / R1, r = t - l * R1;
+      const float2* Y = fft_sm + l * row_ex<R1, R2>() + r * (R2 + 1);
+      float2 u[R2];
 #pragma unroll
-    for (int n2 = 0; n2 < R2; ++n2) u[n2] = Y[n2];
-    fft_phase3<R2, false>(u);
-    float2* Z = Zs + l * row_z(M) + r;
+      for (int n2 = 0; n2 < R2; ++n2) u[n2] = Y[n2];
+      fft_phase3<R2, false>(u);
+      float2* Z = Zs + l * row_z(M) + r;
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) Z[R1 * k2] = u[k2];
-  }
-  __syncthreads();
-  constexpr int H = M / 2;
-#pragma unroll
-  for (int q = 0; q < (L * H + NT - 1) / NT; ++q) {
-    const int m = t + q * NT, l = m / H, k = m - l * H;
-    if (l >= L) break;
-    const float2* Z = Zs + l * row_z(M);
-    float2* out = modes + (row0 + l) * S;
-    if (k == 0) {
-      // X[0] and X[M] from Z[0], X[M/2] from Z[M/2] (W_N^{M/2} = -i)
-      const float2 a = Z[0], c = Z[H];
-      out[0] = make_float2(2.f * (a.x + a.y), 0.f);
-      out[M] = make_float2(2.f * (a.x - a.y), 0.f);
-      out[H] = make_float2(2.f * c.x, -2.f * c.y);
-    } else {
-      const float2 a = Z[k], b = Z[M - k];
-      const float2 e = make_float2(a.x + b.x, a.y - b.y);
-      const float2 o = cmul(make_float2(a.y + b.y, b.x - a.x), __ldg(&twN[k]));
-      out[k] = make_float2(e.x + o.x, e.y + o.y);
-      out[M - k] = make_float2(e.x - o.x, o.y - e.y);
+      for (int k2 = 0; k2 < R2; ++k2) Z[R1 * k2] = u[k2];
     }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < (L * H + NT - 1) / NT; ++q) {
+      const int m = t + q * NT, l = m / H, k = m - l * H;
+      if (l >= L) break;
+      const float2* Z = Zs + l * row_z(M);
+      float2* out = modes + (row0 + l) * S;
+      if (k == 0) {
+        // X[0] and X[M] from Z[0], X[M/2] from Z[M/2] (W_N^{M/2} = -i)
+        const float2 a = Z[0], c = Z[H];
+        out[0] = make_float2(2.f * (a.x + a.y), 0.f);
+        out[M] = make_float2(2.f * (a.x - a.y), 0.f);
+        out[H] = make_float2(2.f * c.x, -2.f * c.y);
+      } else {
+        const float2 a = Z[k], b = Z[M - k];
+        const float2 e = make_float2(a.x + b.x, a.y - b.y);
+        const float2 o = cmul(make_float2(a.y + b.y, b.x - a.x), __ldg(&twN[k]));
+        out[k] = make_float2(e.x + o.x, e.y + o.y);
+        out[M - k] = make_float2(e.x - o.x, o.y - e.y);
+      }
+    }
+  };
+  if constexpr (AGAIN) {
+    for (unsigned block = blockIdx.x; block < N * N / L; block += gridDim.x) {
+      rows(block);
+      __syncthreads();  // the buffers are free for the next rows
+    }
+    const ff w = warp_sum_ff(ff{acc.hi, acc.lo});
+    if ((t & 31) == 0) s_part[t >> 5] = w;
+    __syncthreads();
+  } else {
+    rows(blockIdx.x);
   }
   if (t == 0) {
     ff p = s_part[0];
@@ -243,7 +288,11 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_rfft_ro
     double a = 0.0;
     for (unsigned i = t; i < gridDim.x; i += NT) a += __ldcg(&partials[i]);
     a = block_sum(a);
-    if (t == 0) *inv_mean = (float)((double)N * N * N / a);
+    if (t == 0) {
+      const double mean = a / ((double)N * N * N), green = -coef / mean;
+      scale->green = (float)green;
+      if (!AGAIN) scale->factor = fft_factor(mean, green);
+    }
   }
 }
 
@@ -261,6 +310,7 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_rfft_ro
   const long long row0 = (long long)blockIdx.x * L;
   float2* Zs = fft_sm + L * row_ex<R1, R2>();
   constexpr int H = M / 2;
+  after_previous_pass();
 #pragma unroll
   for (int q = 0; q < (L * H + NT - 1) / NT; ++q) {
     const int m = t + q * NT, l = m / H, k = m - l * H;
@@ -326,12 +376,13 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_rfft_ro
 template <int R1, int R2, bool INV, bool GREEN>
 __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_fft_cols(float2* __restrict__ data, int TC, long long stride_axis,
                                                              long long stride_other, const float2* __restrict__ twN,
-                                                             const float* __restrict__ s2, float coef,
-                                                             const float* __restrict__ inv_mean) {
+                                                             const float* __restrict__ s2,
+                                                             const FftScale* __restrict__ scale) {
   extern __shared__ float2 fft_sm[];
   const int c = threadIdx.x % TC, r = threadIdx.x / TC;
   constexpr int N = R1 * R2, M = N / 2;
   const bool last = (int)blockIdx.x * TC == M;
+  after_previous_pass();
   if (last && (int)blockIdx.y * TC >= N) return;
   const int z = last ? M : blockIdx.x * TC + c;
   const int o = last ? blockIdx.y * TC + c : blockIdx.y;
@@ -357,7 +408,7 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R1, R2>()) k_fft_col
     __syncthreads();  // every phase-3 read of the exchange buffer is done
     if (r < R1) {
       const float sc = s2[o] + s2[z];
-      const float cf = -coef * *inv_mean;  // delta = rho / mean - 1, whose constant drops out at k = 0
+      const float cf = scale->green;  // delta = rho / mean - 1, whose constant drops out at k = 0
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) {
         const float K2 = s2[r + R1 * k2] + sc;
@@ -388,7 +439,7 @@ struct FftPlan {
   float2* tw = nullptr;         // W_N^m, m < N; then W_M^{n2 k1} at k1 F2 + n2 and at k1 F1 + n2 (M = N/2 = F1 F2)
   float* s2 = nullptr;
   double* partials = nullptr;   // one per CTA of the forward rows pass
-  float* inv_mean = nullptr;    // N^3 over the density's sum
+  FftScale* scale = nullptr;    // from the forward rows pass
   unsigned* ticket = nullptr;   // CTAs of the forward rows pass that have finished (0 between calls)
 };
 
@@ -397,7 +448,7 @@ static void free_plan(FftPlan* p) {
   cudaFree(p->tw);
   cudaFree(p->s2);
   cudaFree(p->partials);
-  cudaFree(p->inv_mean);
+  cudaFree(p->scale);
   cudaFree(p->ticket);
   delete p;
 }
@@ -424,7 +475,7 @@ static int fft_plan(int N, FftPlan** out) {
             cudaMalloc(&p->tw, 2 * (size_t)N * sizeof(float2)) == cudaSuccess &&
             cudaMalloc(&p->s2, (size_t)N * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&p->partials, (size_t)N * N * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&p->inv_mean, sizeof(float)) == cudaSuccess &&
+            cudaMalloc(&p->scale, sizeof(FftScale)) == cudaSuccess &&
             cudaMalloc(&p->ticket, sizeof(unsigned)) == cudaSuccess &&
             cudaMemset(p->ticket, 0, sizeof(unsigned)) == cudaSuccess;
   if (ok) {
@@ -476,6 +527,25 @@ void release_fft_plans() {
 
 static bool pow2_mesh(int N) { return N >= 8 && N <= 1024 && (N & (N - 1)) == 0; }
 
+// Launch of a pass that starts with after_previous_pass.
+template <typename... P, typename... A>
+static cudaError_t launch_pass(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+// CTAs of the second forward rows pass: four an SM.
+constexpr unsigned kAgainCtas = 4 * 152;
+
 // The five passes for N = R1 R2 (columns) and N/2 = F1 F2 (forward rows; the
 // inverse swaps the two, so that its stores are runs of the larger factor).
 // Columns kernel: TC = 256/T z modes per tile (at most N/2).  Dynamic shared
@@ -491,8 +561,8 @@ static int poisson_passes(const float* rho, float* phi, double coef, const FftPl
   const size_t cols_smem = (size_t)N * TC * sizeof(float2);
   static bool attr_set[64] = {};  // per device: the opt-in above 48 KB, once
   if (p->device < 64 && !attr_set[p->device]) {
-    MG_CUDA_TRY(cudaFuncSetAttribute(k_rfft_rows_fwd<F1, F2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)fwd_smem));
+    for (auto kern : {k_rfft_rows_fwd<F1, F2, false>, k_rfft_rows_fwd<F1, F2, true>})
+      MG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem));
     MG_CUDA_TRY(cudaFuncSetAttribute(k_rfft_rows_inv<F2, F1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)inv_smem));
     MG_CUDA_TRY(cudaFuncSetAttribute(k_fft_cols<R1, R2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -507,16 +577,22 @@ static int poisson_passes(const float* rho, float* phi, double coef, const FftPl
   const dim3 cols_grid(M / TC + 1, N);
   const long long sy = S, sx = (long long)N * S;
   prof_begin(PC_POISSON_FFT, st, 40.0 * n3);
-  k_rfft_rows_fwd<F1, F2><<<rows_grid, L * F2, fwd_smem, st>>>(rho, p->buf, (uintptr_t)rho % 8 == 0, p->tw, p->tw + N,
-                                                               p->partials, p->ticket, p->inv_mean);
-  k_fft_cols<R1, R2, false, false><<<cols_grid, TC * T, cols_smem, st>>>(p->buf, TC, sy, sx, p->tw, p->s2, 0.f, nullptr);
-  k_fft_cols<R1, R2, false, true><<<cols_grid, TC * T, cols_smem, st>>>(p->buf, TC, sx, sy, p->tw, p->s2, (float)coef,
-                                                                        p->inv_mean);
-  k_fft_cols<R1, R2, true, false><<<cols_grid, TC * T, cols_smem, st>>>(p->buf, TC, sy, sx, p->tw, p->s2, 0.f, nullptr);
-  k_rfft_rows_inv<F2, F1><<<rows_grid, L * F2, inv_smem, st>>>(p->buf, phi, (uintptr_t)phi % 8 == 0,
-                                                               (float)(0.5 / (double)n3), p->tw, p->tw + N + M);
+  const unsigned again_grid = rows_grid < kAgainCtas ? rows_grid : kAgainCtas;
+  const bool pairs = (uintptr_t)rho % 8 == 0;
+  k_rfft_rows_fwd<F1, F2, false><<<rows_grid, L * F2, fwd_smem, st>>>(rho, p->buf, pairs, coef, p->tw, p->tw + N,
+                                                                      p->partials, p->ticket, p->scale);
+  MG_CUDA_TRY(launch_pass(k_rfft_rows_fwd<F1, F2, true>, again_grid, L * F2, fwd_smem, st, rho, p->buf, pairs, coef, p->tw,
+                          p->tw + N, p->partials, p->ticket, p->scale));
+  MG_CUDA_TRY(launch_pass(k_fft_cols<R1, R2, false, false>, cols_grid, TC * T, cols_smem, st, p->buf, TC, sy, sx, p->tw,
+                          p->s2, nullptr));
+  MG_CUDA_TRY(launch_pass(k_fft_cols<R1, R2, false, true>, cols_grid, TC * T, cols_smem, st, p->buf, TC, sx, sy, p->tw,
+                          p->s2, p->scale));
+  MG_CUDA_TRY(launch_pass(k_fft_cols<R1, R2, true, false>, cols_grid, TC * T, cols_smem, st, p->buf, TC, sy, sx, p->tw,
+                          p->s2, nullptr));
+  MG_CUDA_TRY(launch_pass(k_rfft_rows_inv<F2, F1>, rows_grid, L * F2, inv_smem, st, p->buf, phi, (uintptr_t)phi % 8 == 0,
+                          (float)(0.5 / (double)n3), p->tw, p->tw + N + M));
   prof_end(st);
-  note_launch(5);
+  note_launch(6);
   MG_CUDA_TRY(cudaGetLastError());
   return MGGLAM_OK;
 }
