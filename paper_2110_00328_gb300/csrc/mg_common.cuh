@@ -80,23 +80,27 @@ struct FloatFloat {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-// The block's sum in thread 0: the warps' sums by two-sums, then theirs in FP64 -- five
-// FP64 additions of one warp instead of one warp's and eight times five (2432 blocks: 6 us
-// of the FP64 pipe).
+// float -> double, exact; normal numbers by bits, without the conversion, which is an
+// instruction of the 1/64-rate FP64 pipe.
+__device__ __forceinline__ double f2d_exact(float f) {
+  const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+  return (double)f;
+}
+
+// The block's sum (of at most kThreads threads) in thread 0, in FP64, whose range and 53
+// bits the sum needs: one warp adds the threads' values, 2 kThreads / 32 FP64 additions
+// an SM sub-partition serves once instead of the five of every warp's shuffles.
 __device__ __forceinline__ double block_sum(FloatFloat v) {
-  __shared__ double sh[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    const float hi = __shfl_down_sync(0xffffffffu, v.hi, o), lo = __shfl_down_sync(0xffffffffu, v.lo, o);
-    v.add(hi);
-    v.lo += lo;
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ float2 sh[kThreads];
+  const int t = threadIdx.x;
   __syncthreads();
-  if (lane == 0) sh[w] = v.value();
+  sh[t] = make_float2(v.hi, v.lo);
   __syncthreads();
   double s = 0.0;
-  if (w == 0) {
-    s = lane < (int)((blockDim.x + 31) >> 5) ? sh[lane] : 0.0;
+  if (t < 32) {
+    for (int i = t; i < (int)blockDim.x; i += 32) s += f2d_exact(sh[i].x) + f2d_exact(sh[i].y);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   }
   return s;
