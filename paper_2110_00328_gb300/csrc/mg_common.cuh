@@ -80,19 +80,29 @@ struct FloatFloat {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-// float -> double, exact; normal numbers by bits, without the conversion, which is an
-// instruction of the 1/64-rate FP64 pipe.
-__device__ __forceinline__ double f2d_exact(float f) {
+// float -> double, exact; normal numbers and zeros by bits, without the conversion, which
+// is an instruction of the 1/64-rate FP64 pipe.
+__device__ __forceinline__ bool f2d_by_bits(float f) {
+  const unsigned a = __float_as_uint(f) & 0x7fffffffu;
+  return a - 0x00800000u < 0x7f000000u || a == 0u;
+}
+__device__ __forceinline__ double f2d_of_bits(float f) {
   const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
-  if (a - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
-  return (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u)), (int)(b << 29));
+}
+// (a call for the other numbers: as an expression the compiler converts every value and selects)
+static __device__ __noinline__ double f2d_call(float f) { return (double)f; }
+__device__ __forceinline__ double f2d_exact(float f) {
+  if (f2d_by_bits(f)) return f2d_of_bits(f);
+  return f2d_call(f);
 }
 
-// The block's sum (of at most kThreads threads) in thread 0, in FP64, whose range and 53
-// bits the sum needs: one warp adds the threads' values, 2 kThreads / 32 FP64 additions
-// an SM sub-partition serves once instead of the five of every warp's shuffles.
+// The sum of a block of kThreads threads in thread 0, in FP64, whose range and 53 bits
+// the sum needs: one warp adds the threads' values, two FP64 additions a value of its
+// lanes' eight, instead of the five of every warp's shuffles (k_sum_f32 of a 128^3 mesh
+// 9.2 us; 14.6 by shuffles in FP64).
 __device__ __forceinline__ double block_sum(FloatFloat v) {
+  constexpr int P = kThreads / 32;
   __shared__ float2 sh[kThreads];
   const int t = threadIdx.x;
   __syncthreads();
@@ -100,7 +110,22 @@ __device__ __forceinline__ double block_sum(FloatFloat v) {
   __syncthreads();
   double s = 0.0;
   if (t < 32) {
-    for (int i = t; i < (int)blockDim.x; i += 32) s += f2d_exact(sh[i].x) + f2d_exact(sh[i].y);
+    float2 x[P];
+    bool bits = true;
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      x[i] = sh[t + 32 * i];
+      bits = bits && f2d_by_bits(x[i].x) && f2d_by_bits(x[i].y);
+    }
+    double l = 0.0;
+    if (bits) {
+#pragma unroll
+      for (int i = 0; i < P; ++i) s += f2d_of_bits(x[i].x), l += f2d_of_bits(x[i].y);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < P; ++i) s += (double)sh[t + 32 * i].x, l += (double)sh[t + 32 * i].y;
+    }
+    s += l;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   }
   return s;
