@@ -38,15 +38,15 @@ namespace mg {
 
 // ---- per-cell coefficients from the converged field ----
 
-// 1 / x to about one ulp: FP32 seed, two Newton refinements (four FP64 instructions,
-// where a division takes twice that on a pipe of 1/64 of the FP32 rate); outside
+// 1 / x to about half an ulp: FP32 seed y of relative error e <= 2^-22 and the first
+// terms of 1 / (1 - e) = 1 + e + e^2 + ..., which leave e^3 (three FP64 instructions,
+// where a division takes three times that on a pipe of 1/64 of the FP32 rate); outside
 // the range of the seed the division.
 __device__ __forceinline__ double rcp_fast(double x) {
   const float xf = d2f_bits(x), ax = fabsf(xf);
   if (!(ax > 1e-30f && ax < 1e30f)) return 1.0 / x;
-  double y = f2d_bits(frcp(xf));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
+  const double y = f2d_bits(frcp(xf)), e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
 // m64, m32 = mass; rhs = sigma * g (FP64); dinv = 1 / (6 kh + m), the inverse
@@ -769,36 +769,32 @@ __global__ void __launch_bounds__(kThreads) k_adj_apply(int n, double s, double*
 // dl/d delta = gam lambda with gam = -dN/d delta (f(R): -Om/a; symmetron msym
 // (a*/a)^3 u), and partial sums of lambda tq with tq = -dN/d theta (f(R):
 // K/((n+1)u)) and of (dl/d delta_i) rho_i, the term the mean-1 normalisation of the
-// density adds to the gradient with respect to the caller's rho.  The two sums'
-// terms are float-float (48 bits of FP64 inputs, in FP32 instructions), their sums
-// FP64 from a block on.
+// density adds to the gradient with respect to the caller's rho.  Terms and sums in
+// FP64, six instructions of its pipe a cell, which bound it (512^3: 1.4 ms).
 template <int K>
-__global__ void __launch_bounds__(kThreads) k_adj_outputs(ModelDev m, long long n3, int ex,
-                                                          const double* __restrict__ lam,
+__global__ void __launch_bounds__(kThreads) k_adj_outputs(ModelDev m, long long n3, const double* __restrict__ lam,
                                                           const double* __restrict__ u,
                                                           const float* __restrict__ rho32,
                                                           double* __restrict__ grad_rho,
                                                           double* __restrict__ partials,
                                                           double* __restrict__ partials2) {
-  ffacc acc = {0.f, 0.f}, acc2 = {0.f, 0.f};
+  double acc = 0.0, acc2 = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x) {
-    const double lc = lam[t];
-    const ff l = ff_from_double_scaled(lc, ex);
+    double g;
     if constexpr (is_fr(K)) {
-      grad_rho[t] = -m.om_a * lc;
-      acc_add(acc, ff_div(l, ff_from_double(u[t])));
-      acc_add(acc2, ff_mul_f(l, rho32[t]));
+      g = -m.om_a * lam[t];
+      acc = fma(lam[t], rcp_fast(u[t]), acc);
     } else {
-      const double uc = u[t];
-      grad_rho[t] = m.msym * m.rat3 * uc * lc;
-      acc_add(acc2, ff_mul_f(ff_mul(l, ff_from_double(uc)), rho32[t]));
+      g = m.msym * m.rat3 * u[t] * lam[t];
     }
+    grad_rho[t] = g;
+    acc2 = fma(g, f2d_exact(rho32[t]), acc2);
   }
-  const double a = block_sum((double)acc.s + (double)acc.e);
-  if (threadIdx.x == 0) partials[blockIdx.x] = is_fr(K) ? ldexp(a, -ex) * (m.K / (K + 1)) : 0.0;
-  const double a2 = block_sum((double)acc2.s + (double)acc2.e);
-  if (threadIdx.x == 0) partials2[blockIdx.x] = ldexp(a2, -ex) * (is_fr(K) ? -m.om_a : m.msym * m.rat3);
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = is_fr(K) ? acc * (m.K / (K + 1)) : 0.0;
+  acc2 = block_sum(acc2);
+  if (threadIdx.x == 0) partials2[blockIdx.x] = acc2;
 }
 
 // Chain rule through delta = rho / mu - 1, mu = sum(rho) / N^3:
@@ -1079,9 +1075,7 @@ int solve_adjoint(const mgglam_params* prm, double a, const double* field, const
   const double bnorm = sqrt(w->h_scal[0] / (double)n3);
   const double snorm = bnorm > 0.0 ? bnorm : 1.0;
   double eps = bnorm / snorm;
-  // lambda is of the size of rhs / kappa
-  const int unit = bnorm > 0.0 && isfinite(bnorm) ? -ilogb(bnorm / m.c2) : 0;
-  if (ffr) ex = unit;
+  if (ffr && bnorm > 0.0 && isfinite(bnorm)) ex = -ilogb(bnorm / m.c2);  // lambda is of the size of rhs / kappa
   mgglam_stats local;
   mgglam_stats* S = stats ? stats : &local;
   memset(S, 0, sizeof(*S));
@@ -1119,8 +1113,8 @@ int solve_adjoint(const mgglam_params* prm, double a, const double* field, const
   }
   if (outer == 0) MG_CUDA_TRY(cudaMemsetAsync(w->lam, 0, (size_t)n3 * 8, st));  // no correction was applied
   const int go = grid_for(n3);
-  MG_ADJ_DISPATCH(m.kind, (k_adj_outputs<KK><<<go, kThreads, 0, st>>>(m, n3, unit, w->lam, field, rho, grad_rho,
-                                                                      w->partials, w->partials2)));
+  MG_ADJ_DISPATCH(m.kind, (k_adj_outputs<KK><<<go, kThreads, 0, st>>>(m, n3, w->lam, field, rho, grad_rho, w->partials,
+                                                                      w->partials2)));
   k_adj_finalize<<<1, 1024, 0, st>>>(w->partials, w->partials2, go, w->scal);
   note_launch(1);
   if (grad_rho_raw) {
