@@ -91,10 +91,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_setup(ModelDev m, int n, float
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const long long o = SPLIT ? (long long)(c0 ^ c) * H + (long long)row * h + q : t + c;
-        const float mf = d2f_bits(mass[c]);
+        const float mf = d2f_nearest(mass[c]);
         m32[o] = mf;
         dinv[o] = 1.f / (6.f * kh + mf);
-        b[o] = d2f_bits(r[c]);
+        b[o] = d2f_nearest(r[c]);
       }
     }
   }

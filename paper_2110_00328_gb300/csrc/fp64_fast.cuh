@@ -10,19 +10,31 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "float_bits.h"
 #include "mg_model.cuh"
 #include "sweep32.cuh"
 
 namespace mg {
 
-// double -> float by bits, truncated (relative error below 2^-23): 0 below
-// 2^-126, NaN from 2^128 on (and for inf and NaN).
+// double -> float by bits, truncated (relative error below 2^-23), for seeds and
+// Newton steps: 0 below 2^-126, NaN from 2^128 on (and for inf and NaN).
 __device__ __forceinline__ float d2f_bits(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
   const unsigned a = hi & 0x7fffffffu;
   const unsigned m = __funnelshift_l(lo, a, 3) - (896u << 23);
   const unsigned r = a < (897u << 20) ? 0u : (a >= (1151u << 20) ? 0x7fffffffu : m);
   return __uint_as_float(r | (hi & 0x80000000u));
+}
+
+// double -> float as the conversion instruction rounds it: by bits where the result is
+// zero or normal, by the instruction elsewhere (a call: as an expression the compiler
+// converts every value and selects, 11 us of a CQ residual's 58 at 128^3).
+static __device__ __noinline__ float d2f_call(double d) { return (float)d; }
+__device__ __forceinline__ float d2f_nearest(double d) {
+  bool ok;
+  const unsigned r = d2f_nearest_bits((unsigned)__double2hiint(d), (unsigned)__double2loint(d), &ok);
+  if (ok) return __uint_as_float(r);
+  return d2f_call(d);
 }
 
 // float -> double by bits, exact for normal numbers; 0 and subnormals give 0

@@ -621,11 +621,11 @@ __device__ __forceinline__ double cq_residual_tile(const ModelDev& m, const CqSe
     const double uc = s_w[sl][cc];
     const double L = s_w[sm][cc] + s_w[sp][cc] + s_w[sl][cc - PK] + s_w[sl][cc + PK] + s_w[sl][cc - 1] +
                      s_w[sl][cc + 1];
-    const float uf = SERIES ? d2f_bits(uc) : (float)uc;
+    const float uf = SERIES ? d2f_nearest(uc) : (float)uc;
     double v;
     if constexpr (SERIES) {
       const double lap = fma(-6.0, uc, L);
-      const double sc = fma(cq1, f2d_bits(rho[g]), m.cq_src);
+      const double sc = fma(cq1, f2d_exact(rho[g]), m.cq_src);
       const float d = uf * q.d;
       if (fabsf(d) <= kCqSmall) {
         const float rest = q.lf * uf * d * fmaf(d, fmaf(d, q.r4, q.r3), q.r2);
@@ -638,7 +638,7 @@ __device__ __forceinline__ double cq_residual_tile(const ModelDev& m, const CqSe
       const double x = m.phibar + uc / m.c2;
       v = (L - 6.0 * uc) - m.cq_src * (E * src[g] - 1.0) + m.cq_pot * (pow(x, -1.0 - m.alpha) - m.pot0);
     }
-    const float tv = SERIES ? -d2f_bits(v) : (float)(-v);
+    const float tv = SERIES ? -d2f_nearest(v) : (float)(-v);
     const size_t o = SPLIT ? (size_t)split_idx(n, i, jg, kg) : g;
     ub[o] = uf;
     tau[o] = tv;
