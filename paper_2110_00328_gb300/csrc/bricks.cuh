@@ -10,7 +10,6 @@ namespace mg {
 constexpr int kBrickI = 8, kBrickJ = 8, kBrickK = 32;  // particles
 
 constexpr long long kBrickBlocks = 3000;
-constexpr int kBrickOther = 16384;  // blocks of the single-particle kernel launched beside
 
 // The bricks of an M x M x ni array; blocks = 0: not taken.
 struct BrickGrid {
@@ -19,13 +18,15 @@ struct BrickGrid {
 };
 
 // np particles (a multiple of M^2; M = lattice, or 0: in no such order) go by bricks from
-// 3000 bricks (192^3 particles) and half a particle a cell on -- the window of a sparser
+// 3000 bricks (177^3 particles) and half a particle a cell on -- the window of a sparser
 // lattice's brick covers fewer of its particles -- in a mesh of at least the window's
 // longest side.  Fewer bricks are a few waves of CTAs with a last one that is nearly
-// empty, and pay the two extra launches (10 us).  Measured without those (singles /
-// bricks, us; cells, particles): deposit 128^3, 104^3 45.4 / 49.2; 128^3, 128^3 63.5 /
-// 55.1; 192^3, 192^3 183 / 144; 240^3, 192^3 225 / 187; 322^3, 256^3 529 / 415.  Gather
-// 34.9 / 39.6; 45.1 / 43.1; 142 / 119; 182 / 154; 463 / 406.
+// empty.  Measured (singles / bricks, us, whole calls; cells, particles): deposit 128^3,
+// 177^3 121 / 112; 176^3, 177^3 161 / 134; 192^3, 185^3 190 / 153; 192^3, 192^3 204 / 154;
+// 240^3, 192^3 248 / 199; 320^3, 256^3 573 / 446; gather, in the same order but for the
+// first (gather_bricks), 132 / 112; 153 / 128; 160 / 131; 205 / 168; 505 / 375.  Below, the
+// kernels alone: deposit 128^3, 104^3 45.4 / 49.2; 128^3, 128^3 63.5 / 55.1; gather 34.9 /
+// 39.6; 45.1 / 43.1.
 static inline BrickGrid brick_grid(long long np, long long lattice, int N, int window) {
   const long long M = lattice, ni = M > 0 ? np / (M * M) : 0;
   const long long nbj = (M + kBrickJ - 1) / kBrickJ, nbk = (M + kBrickK - 1) / kBrickK,
@@ -47,8 +48,9 @@ static inline long long lattice_side(long long np) {
 // the first.  By bricks particles in no order take longer than by singles (shuffled 256^3:
 // the deposit 1398 against 1256 us, the gather, whose staging kernel keeps fewer warps,
 // 2598 against 1645), so both kernels are launched and the one not meant returns at once.
-static __global__ void __launch_bounds__(256) k_brick_probe(const float* __restrict__ pos, int N, BrickGrid G,
-                                                            int* __restrict__ by_bricks) {
+// One block of 256 threads of a kernel that runs before them asks, beside its own work.
+static __device__ __forceinline__ void brick_probe(const float* __restrict__ pos, int N, const BrickGrid& G,
+                                                   int* __restrict__ by_bricks) {
   const unsigned b = (unsigned)((unsigned long long)threadIdx.x * G.blocks / 256);
   const int bk = b % G.nbk, bj = b / G.nbk % G.nbj, bi = b / G.nbk / G.nbj;
   const int i = bi * kBrickI, j = bj * kBrickJ, k = bk * kBrickK;
@@ -65,6 +67,37 @@ static __global__ void __launch_bounds__(256) k_brick_probe(const float* __restr
   }
   const int n = __syncthreads_count(in);
   if (threadIdx.x == 0) *by_bricks = n >= 128;
+}
+
+static __global__ void __launch_bounds__(256) k_brick_probe(const float* __restrict__ pos, int N, BrickGrid G,
+                                                            int* __restrict__ by_bricks) {
+  brick_probe(pos, N, G, by_bricks);
+}
+
+// The single-particle kernel is a programmatic dependent launch of the brick kernel,
+// whose blocks call next_may_start as they begin: its own blocks, which need nothing of
+// the brick kernel's, then come and go beside the last bricks.  Whether they are meant
+// was written before the brick kernel began.  Block 0 stays for the brick kernel's end,
+// so that what follows in the stream follows both.
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ bool left_to_bricks(const int* by_bricks) {
+  if (!by_bricks) return false;
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  return *by_bricks;
+}
+
+template <typename... P, typename... A>
+static cudaError_t launch_beside_bricks(void (*kern)(P...), unsigned blocks, int threads, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
 // The gradients of a mesh scalar at lattice-ordered particles (cic_grad), brick by brick.

@@ -82,7 +82,7 @@ template <typename IT>
 __global__ void __launch_bounds__(kThreads) k_deposit_fixed(const float* __restrict__ pos, long long np, int N,
                                                             unsigned long long* __restrict__ acc,
                                                             const int* by_bricks) {
-  if (by_bricks && *by_bricks) return;
+  if (left_to_bricks(by_bricks)) return;
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < np; base += stride) {
@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(kThreads) k_deposit_fixed(const float* __restr
 // 2048 weights of at most 2^32 fit.  A particle outside the window (1% of 256^3
 // Zel'dovich particles of pixel sigma 1.5) goes to the mesh directly, so any
 // positions are taken; the integer sums are the same in any order.
-// Measured (those particles, the whole call): 470 us before, 325 by this kernel alone, 343
-// with k_brick_probe and the other kernel's launch; pixel sigma 5: 652 and 474.  Issue slots (69%) and the 16 shared atomics a
+// Measured (those particles, the whole call): 470 us before, 335 with both kernels'
+// launches; pixel sigma 5: 654 and 469.  Issue slots (69%) and the 16 shared atomics a
 // particle (L1 68%) share the bound; 32-bit sums with a carry (8 atomics and few
 // carries a particle) are no faster, nor are two CTAs an SM (348).
 constexpr int kWinI = 14, kWinJ = 14, kWinK = 40;               // cells
@@ -174,17 +174,13 @@ __device__ __noinline__ void deposit_direct(const float* __restrict__ x, int N, 
 }
 
 template <typename IT>
-__global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float* __restrict__ pos, int M, int ni,
-                                                                     int nbj, int nbk, int N,
-                                                                     unsigned long long* __restrict__ acc,
-                                                                     const int* by_bricks) {
-  if (!*by_bricks) return;
+__device__ __forceinline__ void deposit_brick(unsigned b, const float* __restrict__ pos, int M, int ni, int nbj, int nbk,
+                                              int N, unsigned long long* __restrict__ acc) {
   extern __shared__ __align__(16) unsigned win[];  // low words, then high words; cleared 16 bytes at a time
   __shared__ int s_sum[4], s_nout;
   __shared__ unsigned short s_out[kBrickOut];  // particles outside the window
   const int t = threadIdx.x;
-  const unsigned b = blockIdx.x, bij = b / (unsigned)nbk, bk = b - bij * nbk, bi = bij / (unsigned)nbj,
-                 bj = bij - bi * nbj;
+  const unsigned bij = b / (unsigned)nbk, bk = b - bij * nbk, bi = bij / (unsigned)nbj, bj = bij - bi * nbj;
   const int i0 = bi * kBrickI + t / (kBrickJ * kBrickK), j0 = bj * kBrickJ + (t / kBrickK) % kBrickJ,
             k0 = bk * kBrickK + t % kBrickK;
   const float* brick = pos + 3 * (((long long)bi * kBrickI * M + bj * kBrickJ) * M + bk * kBrickK);  // its first particle
@@ -279,27 +275,76 @@ __global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float
   }
 }
 
+// Three CTAs an SM for the whole kernel, which take the bricks in turns: where the
+// particles are in no order 456 CTAs come and go in a microsecond, one a brick in five
+// (256^3, 192^3: 1270 and 278 us a call, 1259 and 276 so, 1259 and 274 by singles alone).
+constexpr unsigned kBrickCtas = 3 * 152;
+template <typename IT>
+__global__ void __launch_bounds__(kBrickThreads, 3) k_deposit_bricks(const float* __restrict__ pos, int M, int ni,
+                                                                     int nbj, int nbk, unsigned bricks, int N,
+                                                                     unsigned long long* __restrict__ acc,
+                                                                     const int* by_bricks) {
+  next_may_start();
+  if (!*by_bricks) return;
+#pragma unroll 1
+  for (unsigned b = blockIdx.x; b < bricks; b += gridDim.x) {
+    deposit_brick<IT>(b, pos, M, ni, nbj, nbk, N, acc);
+    __syncthreads();  // the window is free for the next brick
+  }
+}
+
+// acc <- 0, and brick_probe beside it.
+__global__ void __launch_bounds__(kThreads) k_deposit_clear(unsigned long long* __restrict__ acc, long long n3,
+                                                            const float* __restrict__ pos, int N, BrickGrid b,
+                                                            int* __restrict__ by_bricks) {
+  if (blockIdx.x == 0) brick_probe(pos, N, b, by_bricks);
+  ulonglong2* a = reinterpret_cast<ulonglong2*>(acc);
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3 >> 1;
+       t += (long long)gridDim.x * blockDim.x)
+    a[t] = make_ulonglong2(0ull, 0ull);
+  if ((n3 & 1) && blockIdx.x == 0 && threadIdx.x == 0) acc[n3 - 1] = 0ull;
+}
+
+// Where the deposit's kernels learn whether the particles go by bricks: the word behind
+// acc's N^3.
+static int* deposit_flag(unsigned long long* acc, int N) { return reinterpret_cast<int*>(acc + (long long)N * N * N); }
+
+// Clears acc for np particles, and asks for the deposit's order where it will be in question.
+static int clear_deposit(const float* pos, long long np, long long lattice, int N, unsigned long long* acc,
+                         cudaStream_t st) {
+  const long long n3 = (long long)N * N * N;
+  const BrickGrid b = brick_grid(np, lattice, N, kWinK);
+  if (!b.blocks) {
+    MG_CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)n3 * sizeof(unsigned long long), st));
+    return MGGLAM_OK;
+  }
+  k_deposit_clear<<<stream_grid(n3), kThreads, 0, st>>>(acc, n3, pos, N, b, deposit_flag(acc, N));
+  note_launch(1);
+  MG_CUDA_TRY(cudaGetLastError());
+  return MGGLAM_OK;
+}
+
 // The deposit of np particles on acc, brick by brick (brick_grid; at fewer particles the
 // window's zeroing and flush, four cells a particle, cost more than the atomics they
-// save) or in the order of the array.  lattice: M, or 0.  The word behind acc's N^3 says
-// which of the two (k_brick_probe).
+// save) or in the order of the array.  lattice: M, or 0.  probed: clear_deposit has asked
+// which, of these particles.
 static int launch_deposit(const float* pos, long long np, long long lattice, int N, unsigned long long* acc,
-                          cudaStream_t st) {
+                          bool probed, cudaStream_t st) {
   const BrickGrid b = brick_grid(np, lattice, N, kWinK);
+  // 32-bit cell offsets where the mesh has at most 2^30 cells
+  auto singles = N <= 1024 ? k_deposit_fixed<int> : k_deposit_fixed<long long>;
   if (b.blocks) {
     constexpr int smem = 2 * kWinCells * (int)sizeof(unsigned);
     auto kern = N <= 1024 ? k_deposit_bricks<int> : k_deposit_bricks<long long>;
     MG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    int* by_bricks = reinterpret_cast<int*>(acc + (long long)N * N * N);
-    k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
-    kern<<<b.blocks, kBrickThreads, smem, st>>>(pos, b.M, b.ni, b.nbj, b.nbk, N, acc, by_bricks);
-    (N <= 1024 ? k_deposit_fixed<int> : k_deposit_fixed<long long>)<<<grid_for(np, kThreads, kBrickOther), kThreads, 0,
-                                                                       st>>>(pos, np, N, acc, by_bricks);
-    note_launch(2);
+    int* by_bricks = deposit_flag(acc, N);
+    if (!probed) k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
+    kern<<<b.blocks < kBrickCtas ? b.blocks : kBrickCtas, kBrickThreads, smem, st>>>(pos, b.M, b.ni, b.nbj, b.nbk, b.blocks, N,
+                                                                                      acc, by_bricks);
+    MG_CUDA_TRY(launch_beside_bricks(singles, grid_for(np, kThreads, 1 << 20), kThreads, st, pos, np, N, acc, by_bricks));
+    note_launch(probed ? 1 : 2);
   } else {
-    // 32-bit cell offsets where the mesh has at most 2^30 cells
-    (N <= 1024 ? k_deposit_fixed<int> : k_deposit_fixed<long long>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0,
-                                                                       st>>>(pos, np, N, acc, nullptr);
+    singles<<<grid_for(np, kThreads, 1 << 20), kThreads, 0, st>>>(pos, np, N, acc, nullptr);
   }
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
@@ -341,9 +386,9 @@ int deposit_cic(const float* pos, long long np, int N, float* rho, cudaStream_t 
   int rc = deposit_scratch(N, &acc);
   if (rc) return rc;
   const long long n3 = (long long)N * N * N;
-  MG_CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)n3 * sizeof(unsigned long long), st));
+  if ((rc = clear_deposit(pos, np, lattice_side(np), N, acc, st))) return rc;
   prof_begin(PC_DEPOSIT, st, 12.0 * np);
-  if ((rc = launch_deposit(pos, np, lattice_side(np), N, acc, st))) return rc;
+  if ((rc = launch_deposit(pos, np, lattice_side(np), N, acc, true, st))) return rc;
   prof_end(st);
   prof_begin(PC_DEPOSIT_FINISH, st, 12.0 * n3);
   k_deposit_finish<<<stream_grid(n3), kThreads, 0, st>>>(acc, n3, (double)n3 / (double)np, rho);
@@ -361,9 +406,13 @@ int deposit_cic(const float* pos, long long np, int N, float* rho, cudaStream_t 
 // float-float (FP32 instructions; the exact split of the FP64 field, v - ubar
 // exact to first order, ~48-bit products), which rounds to the same float as
 // FP64 would at 1/64 of FP32's rate; CQ (one product) stays in FP64.
+// Also brick_probe, where b is a grid of bricks.
 template <int K>
-__global__ void k_transform(const double* __restrict__ u, long long n3, double ubar, double beta,
-                            float* __restrict__ T) {
+__global__ void __launch_bounds__(kThreads) k_transform(const double* __restrict__ u, long long n3, double ubar,
+                                                        double beta, float* __restrict__ T,
+                                                        const float* __restrict__ pos, int N, BrickGrid b,
+                                                        int* __restrict__ by_bricks) {
+  if (b.blocks && blockIdx.x == 0) brick_probe(pos, N, b, by_bricks);
   const ff ub = ff_from_double(ubar);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x) {
@@ -384,11 +433,11 @@ __global__ void k_transform(const double* __restrict__ u, long long n3, double u
 
 // One particle per thread (cic_grad: the 32 distinct cells its three central
 // differences at the 8 CIC cells touch).
-template <typename IT>
-__global__ void __launch_bounds__(kThreads) k_gather(const float* __restrict__ T, int N, const float* __restrict__ pos,
-                                                     long long np, float scale, float* __restrict__ force,
-                                                     const int* by_bricks) {
-  if (by_bricks && *by_bricks) return;
+template <typename IT, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_gather(const float* __restrict__ T, int N, const float* __restrict__ pos,
+                                                    long long np, float scale, float* __restrict__ force,
+                                                    const int* by_bricks) {
+  if (left_to_bricks(by_bricks)) return;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < np;
        q += (long long)gridDim.x * blockDim.x) {
     const float3 g = cic_grad<IT>(T, N, pos[3 * q + 0], pos[3 * q + 1], pos[3 * q + 2]);
@@ -399,13 +448,14 @@ __global__ void __launch_bounds__(kThreads) k_gather(const float* __restrict__ T
 }
 
 // The same gather brick by brick (brick_gradients).  Measured (256^3 Zel'dovich
-// particles of pixel sigma 1.5, with the transform's 39 us): 359 us before, 270 by this
-// kernel alone, 289 with k_brick_probe and the other kernel's launch; sigma 3: 604 and 387.
+// particles of pixel sigma 1.5, with the transform's 39 us): 361 us before, 285 with both
+// kernels' launches; sigma 3: 605 and 378.
 template <typename IT, bool QUADS>
 __global__ void __launch_bounds__(kTileThreads, 4) k_gather_bricks(const float* __restrict__ T, int N,
                                                                    const float* __restrict__ pos, BrickGrid b,
                                                                    float scale, float* __restrict__ force,
                                                                    const int* by_bricks) {
+  next_may_start();
   if (!*by_bricks) return;
   brick_gradients<IT, QUADS>(T, N, pos, b, [&](long long p, const float*, float3 g) {
     force[p] = scale * g.x;
@@ -414,26 +464,42 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_gather_bricks(const float* 
   });
 }
 
-// The gather of np particles: brick by brick where the deposit would be, in a mesh of at
-// least the window's longest side.  lattice: as launch_deposit's.
+// Beside the bricks the particles go by blocks of 768 threads (two an SM): fewer that
+// come and go, and they keep more of a warp's lines in L1.  Shuffled 256^3 particles 1598
+// us, 1649 by blocks of 256 alone; ordered ones 283 by bricks with 16384 such blocks
+// beside, 289 with one for every 768 particles.
+constexpr int kWideThreads = 768, kWideBlocks = 16384;
+
+// The gather's bricks: the deposit's, in a mesh of at least the window's longest side,
+// where N np >= 8.4e8.  In a mesh much coarser than the lattice the particles of a warp
+// share their cells, the single-particle kernel finds them in L1, and few bricks are no
+// gain.  Measured (singles / bricks, us; cells, particles): 96^3, 177^3 85 / 88; 128^3,
+// 185^3 98 / 100; 64^3, 216^3 133 / 135; on the other side 160^3, 177^3 115 / 100; 128^3,
+// 192^3 112 / 104; 96^3, 216^3 139 / 137; 64^3, 256^3 213 / 203.
+static BrickGrid gather_bricks(long long np, long long lattice, int N) {
+  return brick_grid(np, (double)N * (double)np >= 8.4e8 ? lattice : 0, N, kTileK);
+}
+
+// The gather of np particles.  lattice, probed: as launch_deposit's (the transform asks).
 static int launch_gather(const float* T, int N, const float* pos, long long np, long long lattice, float scale,
-                         float* force, int* by_bricks, cudaStream_t st) {
-  const BrickGrid b = brick_grid(np, lattice, N, kTileK);
+                         float* force, int* by_bricks, bool probed, cudaStream_t st) {
+  const BrickGrid b = gather_bricks(np, lattice, N);
   if (b.blocks) {
     constexpr int smem = kTileCells * (int)sizeof(float);
     const bool quads = N % 4 == 0;  // T's rows on 16-byte boundaries (the workspace's mesh is)
     auto kern = N <= 1024 ? (quads ? k_gather_bricks<int, true> : k_gather_bricks<int, false>)
                           : (quads ? k_gather_bricks<long long, true> : k_gather_bricks<long long, false>);
     MG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
+    if (!probed) k_brick_probe<<<1, 256, 0, st>>>(pos, N, b, by_bricks);
     kern<<<b.blocks, kTileThreads, smem, st>>>(T, N, pos, b, scale, force, by_bricks);
-    (N <= 1024 ? k_gather<int> : k_gather<long long>)<<<grid_for(np, kThreads, kBrickOther), kThreads, 0, st>>>(
-        T, N, pos, np, scale, force, by_bricks);
-    note_launch(2);
+    auto singles = N <= 1024 ? k_gather<int, kWideThreads> : k_gather<long long, kWideThreads>;
+    MG_CUDA_TRY(launch_beside_bricks(singles, grid_for(np, kWideThreads, kWideBlocks), kWideThreads, st, T, N, pos, np,
+                                     scale, force, by_bricks));
+    note_launch(probed ? 1 : 2);
   } else {
     // 32-bit cell offsets where the mesh has at most 2^30 cells
-    (N <= 1024 ? k_gather<int> : k_gather<long long>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0, st>>>(
-        T, N, pos, np, scale, force, nullptr);
+    (N <= 1024 ? k_gather<int, kThreads> : k_gather<long long, kThreads>)<<<grid_for(np, kThreads, 1 << 20), kThreads, 0,
+                                                                            st>>>(T, N, pos, np, scale, force, nullptr);
   }
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
@@ -459,7 +525,7 @@ int gather_chunk(const ModelDev& m, int kind, const mgglam_params* prm, int N, c
   const float* T = ws->lev[0].ub;
   prof_begin(PC_GATHER, st, 24.0 * np);
   rc = launch_gather(T, N, pos, np, lattice, (float)(force_scale(m, kind, prm) * prefactor), force,
-                     by_bricks_of(ws), st);
+                     by_bricks_of(ws), false, st);
   prof_end(st);
   return rc;
 }
@@ -473,21 +539,23 @@ int gather_force(const ModelDev& m, int kind, int n_fr, const mgglam_params* prm
   float* T = ws->lev[0].ub;  // scratch mesh of N^3 floats
   const long long n3 = (long long)N * N * N;
   const int g = stream_grid(n3);
+  if (lattice < 0) lattice = lattice_side(np);
+  const BrickGrid b = gather_bricks(np, lattice, N);
+  int* by_bricks = by_bricks_of(ws);
   double scale;
   prof_begin(PC_TRANSFORM, st, 12.0 * n3);
   switch (kind) {
-    case KFR0: k_transform<KFR0><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T); break;
-    case KFR1: k_transform<KFR1><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T); break;
-    case KFR2: k_transform<KFR2><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T); break;
-    case KSYM: k_transform<KSYM><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T); break;
-    default: k_transform<KCQ><<<g, kThreads, 0, st>>>(field, n3, 0.0, prm->beta, T); break;
+    case KFR0: k_transform<KFR0><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T, pos, N, b, by_bricks); break;
+    case KFR1: k_transform<KFR1><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T, pos, N, b, by_bricks); break;
+    case KFR2: k_transform<KFR2><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T, pos, N, b, by_bricks); break;
+    case KSYM: k_transform<KSYM><<<g, kThreads, 0, st>>>(field, n3, m.ubar, 0.0, T, pos, N, b, by_bricks); break;
+    default: k_transform<KCQ><<<g, kThreads, 0, st>>>(field, n3, 0.0, prm->beta, T, pos, N, b, by_bricks); break;
   }
   prof_end(st);
   scale = force_scale(m, kind, prm);
   prof_begin(PC_GATHER, st, 24.0 * np + 4.0 * n3);
   note_launch(1);
-  rc = launch_gather(T, N, pos, np, lattice < 0 ? lattice_side(np) : lattice, (float)(scale * prefactor), force,
-                     by_bricks_of(ws), st);
+  rc = launch_gather(T, N, pos, np, lattice, (float)(scale * prefactor), force, by_bricks, true, st);
   prof_end(st);
   return rc;
 }
@@ -551,7 +619,8 @@ int deposit_cic_host(const float* pos_host, float* pos_dev, long long np, int N,
     MG_CUDA_TRY(cudaStreamWaitEvent(st, io->ev[c], 0));
     // a chunk that ends between lattice planes is no lattice
     const long long M = lattice_side(np);
-    if ((rc = launch_deposit(pos_dev + 3 * q0, cnt, M > 0 && q0 % (M * M) == 0 ? M : 0, N, acc, st))) return rc;
+    if ((rc = launch_deposit(pos_dev + 3 * q0, cnt, M > 0 && q0 % (M * M) == 0 ? M : 0, N, acc, false, st)))
+      return rc;
   }
   prof_end(st);
   prof_begin(PC_DEPOSIT_FINISH, st, 12.0 * n3);
@@ -663,8 +732,8 @@ extern "C" int mgglam_deposit_cic_static(const float* pos, long long np, int N, 
   cudaStream_t st = (cudaStream_t)stream;
   const long long n3 = (long long)N * N * N;
   // the array keeps the previous call's sums: clear the part this call uses
-  MG_CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)n3 * sizeof(unsigned long long), st));
-  if ((rc = launch_deposit(pos, np, lattice_side(np), N, acc, st))) return rc;
+  if ((rc = clear_deposit(pos, np, lattice_side(np), N, acc, st))) return rc;
+  if ((rc = launch_deposit(pos, np, lattice_side(np), N, acc, true, st))) return rc;
   k_deposit_finish<<<stream_grid(n3), kThreads, 0, st>>>(acc, n3, (double)n3 / (double)np, rho);
   note_launch(1);
   MG_CUDA_TRY(cudaGetLastError());
