@@ -109,12 +109,11 @@ static cudaError_t launch_beside_bricks(void (*kern)(P...), unsigned blocks, int
 // rows start at multiples of four cells, so that they arrive as 16-byte copies (four
 // times fewer instructions) where N is one too.  A particle outside the window reads
 // the mesh itself, after the others.  The sums are cic_grad's, in its order.
-// More warps matter more than a wider window (the gather's 270 us at 256^3): 16 x 16 x 48
-// cells 274 us, three CTAs an SM 302, 512 threads a CTA 310.
+// More warps matter more than a wider window (the gather's 270 us at 256^3 without other launches): 16 x
+// 16 x 48 cells 274 us, three CTAs an SM 302, 512 threads a CTA 310.
 constexpr int kTileI = 15, kTileJ = 15, kTileK = 48;  // cells
 constexpr int kTileCells = kTileI * kTileJ * kTileK;
-constexpr int kTilePlanes = 1;                        // of a brick at a time
-constexpr int kTileThreads = kTilePlanes * kBrickJ * kBrickK;
+constexpr int kTileThreads = kBrickJ * kBrickK;       // one plane of a brick at a time
 constexpr int kTileOut = 512;
 
 template <typename IT>
@@ -122,8 +121,7 @@ __device__ __noinline__ float3 gradient_direct(const float* T, int N, const floa
   return cic_grad<IT>(T, N, x[0], x[1], x[2]);
 }
 
-// emit(3 q, position of particle q, gradient), once a particle; it may move the particle.
-// QUADS: N % 4 == 0 and T on a 16-byte boundary.
+// emit(3 q, gradient of particle q), once a particle.  QUADS: N % 4 == 0 and T on a 16-byte boundary.
 template <typename IT, bool QUADS, class Emit>
 __device__ __forceinline__ void brick_gradients(const float* __restrict__ T, int N, const float* pos,
                                                 const BrickGrid& G, const Emit& emit) {
@@ -134,14 +132,11 @@ __device__ __forceinline__ void brick_gradients(const float* __restrict__ T, int
   const int M = G.M, ni = G.ni;
   const unsigned b = blockIdx.x, bij = b / (unsigned)G.nbk, bk = b - bij * G.nbk, bi = bij / (unsigned)G.nbj,
                  bj = bij - bi * G.nbj;
-  const int i0 = bi * kBrickI + t / (kBrickJ * kBrickK), j0 = bj * kBrickJ + (t / kBrickK) % kBrickJ,
-            k0 = bk * kBrickK + t % kBrickK;
-  const long long brick = ((long long)bi * kBrickI * M + bj * kBrickJ) * M + bk * kBrickK;  // its first particle
-  const long long mine = ((long long)i0 * M + j0) * M + k0;                                 // this thread's first
-  const long long plane = (long long)kTilePlanes * M * M;                                   // and the next ones' distance
-  const int mp = j0 < M && k0 < M && i0 < ni
-                     ? min(kBrickI / kTilePlanes, (ni - i0 + kTilePlanes - 1) / kTilePlanes)
-                     : 0;  // this thread's particles
+  const int i0 = bi * kBrickI, j0 = bj * kBrickJ + t / kBrickK, k0 = bk * kBrickK + t % kBrickK;
+  const long long brick = ((long long)i0 * M + bj * kBrickJ) * M + bk * kBrickK;  // its first particle
+  const long long mine = ((long long)i0 * M + j0) * M + k0;                       // this thread's first
+  const long long plane = (long long)M * M;                                       // and the next ones' distance
+  const int mp = j0 < M && k0 < M ? min(kBrickI, ni - i0) : 0;                    // this thread's particles
   if (t < 4) s_sum[t] = 0;
   if (t == 4) s_nout = 0;
   __syncthreads();
@@ -212,11 +207,11 @@ __device__ __forceinline__ void brick_gradients(const float* __restrict__ T, int
       const float* at = tile + ((c[0] - 1) * kTileJ + c[1] - 1) * kTileK + c[2] - 1;
       const float3 g =
           cic_grad_core([&](int a, int bb, int cc) { return at[(a * kTileJ + bb) * kTileK + cc]; }, w[0], w[1], w[2]);
-      emit(p, pos + p, g);
+      emit(p, g);
     } else {
       const int q = atomicAdd(&s_nout, 1);
       if (q < kTileOut) s_out[q] = (unsigned short)(t + r * kTileThreads);
-      else emit(p, pos + p, gradient_direct<IT>(T, N, pos + p));
+      else emit(p, gradient_direct<IT>(T, N, pos + p));
     }
   }
   __syncthreads();
@@ -224,7 +219,7 @@ __device__ __forceinline__ void brick_gradients(const float* __restrict__ T, int
     const int x = s_out[q];
     const int i = x / (kBrickJ * kBrickK), j = (x / kBrickK) % kBrickJ, k = x % kBrickK;
     const long long p = 3 * (brick + ((long long)i * M + j) * M + k);
-    emit(p, pos + p, gradient_direct<IT>(T, N, pos + p));
+    emit(p, gradient_direct<IT>(T, N, pos + p));
   }
 }
 

@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_gather_bricks(const float* 
                                                                    const int* by_bricks) {
   next_may_start();
   if (!*by_bricks) return;
-  brick_gradients<IT, QUADS>(T, N, pos, b, [&](long long p, const float*, float3 g) {
+  brick_gradients<IT, QUADS>(T, N, pos, b, [&](long long p, float3 g) {
     force[p] = scale * g.x;
     force[p + 1] = scale * g.y;
     force[p + 2] = scale * g.z;

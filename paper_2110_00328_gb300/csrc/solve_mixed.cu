@@ -147,14 +147,14 @@ __global__ void __launch_bounds__(128) k_residual_restrict32q(LevelF f, int nf, 
 }
 
 // Prolongation: grid (ceil(nf/128), nf / quad_rows(nf) [j], nf/4 [i]).
-template <bool FR, class FL = NatLayout, int QK = -1, bool SECOND_ONLY = false>
+template <bool FR, class FL = NatLayout, int QK = -1>
 __global__ void __launch_bounds__(128) k_prolong_correct32q(int nc, const float* __restrict__ eH,
                                                             const float* __restrict__ Re,
                                                             const float* __restrict__ ub, float* __restrict__ ef,
                                                             unsigned long long* guard,
                                                             float* __restrict__ qf = nullptr) {
   const QuadLane<> ql(2 * nc, blockIdx.y, blockIdx.x, threadIdx.x);
-  prolong_quad<FR, FL, QK, SECOND_ONLY>(nc, eH, Re, ub, ef, blockIdx.z * 4 + threadIdx.y, ql.j, ql.tq, threadIdx.x,
+  prolong_quad<FR, FL, QK>(nc, eH, Re, ub, ef, blockIdx.z * 4 + threadIdx.y, ql.j, ql.tq, threadIdx.x,
                                         guard, qf);
 }
 
