@@ -89,8 +89,8 @@ def measured_peaks():
 # dram__bytes_write.sum of both colour launches of a warm sweep (cycle 6, the
 # path every pass after an inner solve's first sweep takes), from one ncu
 # capture; valid while the kernel's sources hash to the value recorded with it.
-SMOOTHER_TRAFFIC = {"bytes_per_sweep": (134.504192 + 43.464960 + 134.503680 + 38.503680) * 1e6,
-                    "source_sha256_16": "dcdff3862188ebf9"}
+SMOOTHER_TRAFFIC = {"bytes_per_sweep": (134.503936 + 43.439616 + 134.500608 + 38.451200) * 1e6,
+                    "source_sha256_16": "1c9967ae12320cb9"}
 
 
 def smoother_traffic_per_sweep():
