@@ -89,8 +89,8 @@ def measured_peaks():
 # dram__bytes_write.sum of both colour launches of a warm sweep (cycle 6, the
 # path every pass after an inner solve's first sweep takes), from one ncu
 # capture; valid while the kernel's sources hash to the value recorded with it.
-SMOOTHER_TRAFFIC = {"bytes_per_sweep": (134.503936 + 43.439616 + 134.500608 + 38.451200) * 1e6,
-                    "source_sha256_16": "1c9967ae12320cb9"}
+SMOOTHER_TRAFFIC = {"bytes_per_sweep": (134.503168 + 43.262720 + 134.501888 + 38.242048) * 1e6,
+                    "source_sha256_16": "d1a923f202f69069"}
 
 
 def smoother_traffic_per_sweep():

@@ -77,7 +77,6 @@ struct FloatFloat {
     hi = s;
     lo = __fadd_rn(lo, err);
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
 // float -> double, exact; normal numbers and zeros by bits, without the conversion, which

@@ -81,7 +81,7 @@ struct Workspace {
 // SC_FFC: start of the float-float residual constants (48 bytes, mixed path).
 // SC_GUARD holds a 64-bit integer: the positivity-guard replacements of the running solve.
 enum Scalar { SC_MEAN = 0, SC_SUMSQ = 1, SC_SRC = 2, SC_FLAG = 3, SC_GUARD = 4, SC_BRICKS = 5, SC_FFC = 8, SC_COUNT = 16 };
-// SC_BRICKS holds an int: whether the gather's particles go by bricks (k_brick_probe).
+// SC_BRICKS holds an int: whether the gather's particles go by bricks (brick_probe).
 inline int* by_bricks_of(Workspace* ws) { return reinterpret_cast<int*>(ws->scalars + SC_BRICKS); }
 inline unsigned long long* guard_of(Workspace* ws) {
   return reinterpret_cast<unsigned long long*>(ws->scalars + SC_GUARD);
